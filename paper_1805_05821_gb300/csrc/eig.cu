@@ -6,13 +6,11 @@
 //                      U Sigma gives U and Sigma without forming W (Sec. 3.2.2 rank truncation).
 //   project_t/g_kernel G = U_r^T H_m U_r (copy_h_kernel: G = H_m without truncation).
 //   hessenberg_kernel  Householder reduction of G to upper Hessenberg form G = Q Hs Q^T.
-//   hqr_kernel         eigenvalues of Hs by the Francis double-shift QR iteration (single CTA;
-//                      the sequential steps of the EISPACK routine hqr).
-//   vectors_kernel     per eigenvalue: right and left eigenvectors of Hs by inverse iteration
-//                      (LU of Hs - lambda I with adjacent-row pivoting), z = Q z_hs normalised
-//                      (unit norm, largest entry real positive), the amplitude
-//                      c = (w^H b)/(w^H z) with b = beta_11 U_r^T e_1 (Sec. 3.2.4, Eqs.
-//                      exrecon/exreconwrt), the error indicator of Sec. 3.2.3 and y = U_r z.
+//   eig_roots.cu       eigenvalues of Hs by simultaneous iteration, all SMs at work.
+//   hqr_kernel         where that does not apply or converge: the Francis double-shift QR iteration
+//                      (single CTA; the sequential steps of the EISPACK routine hqr).
+//   eig_vectors.cu     per eigenvalue: right and left eigenvectors of Hs by inverse iteration, and
+//                      from them z, the amplitude, the error indicator and y = U_r z.
 //   order_kernel       ordering by |c| (conjugate pairs share the larger |c|), |lambda|, Im.
 //
 // The modes Phi = V y_i are formed by the GEMM in modes.cu.
@@ -80,19 +78,6 @@ __device__ bool wait_neighbours(GridBar *gb, int p, int np, unsigned target, int
   }
   __syncthreads();
   return ok != 0;
-}
-
-__device__ __forceinline__ double block_sum(double v, double *red) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  const int nw = blockDim.x >> 5;
-  for (int i = 0; i < nw; ++i) t += red[i];
-  __syncthreads();
-  return t;
 }
 
 __device__ __forceinline__ int block_max_int(int v, int *red) {
@@ -399,6 +384,7 @@ __global__ void hessenberg_kernel(double *G, int ldg, double *Q, int ldq, const 
 __global__ void hqr_kernel(double *Ag, int lda, const int *isc_in, double *wr, double *wi, int *isc,
                            int smem_elems) {
   const int n = isc_in[ISC_R];
+  if (!isc_in[ISC_QR]) return;
   extern __shared__ double sh[];
   const int tid = threadIdx.x, lane = tid & 31;
   const int T1 = blockDim.x - 32;  // threads outside warp 0
@@ -695,328 +681,6 @@ __global__ void hqr_kernel(double *Ag, int lda, const int *isc_in, double *wr, d
 #undef AA
 }
 
-// ------------------------------------------------------------------------------ vectors
-struct cplx {
-  double re, im;
-};
-__device__ __forceinline__ cplx cmul(cplx a, cplx b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
-__device__ __forceinline__ cplx cconj(cplx a) { return {a.re, -a.im}; }
-__device__ __forceinline__ cplx csub(cplx a, cplx b) { return {a.re - b.re, a.im - b.im}; }
-__device__ __forceinline__ double cabs2(cplx a) { return a.re * a.re + a.im * a.im; }
-__device__ __forceinline__ cplx cdiv(cplx a, cplx b) {
-  // Smith's algorithm
-  if (fabs(b.re) >= fabs(b.im)) {
-    const double r = b.im / b.re, d = b.re + b.im * r;
-    return {(a.re + a.im * r) / d, (a.im - a.re * r) / d};
-  }
-  const double r = b.re / b.im, d = b.re * r + b.im;
-  return {(a.re * r + a.im) / d, (a.im * r - a.re) / d};
-}
-
-// One CTA per eigenvalue with Im >= 0 (the -Im partner of a pair is its conjugate).
-__global__ void vectors_kernel(EigArgs e) {
-  const int r = e.isc[ISC_R];
-  const int m = e.m;
-  const double hlast = *e.hlast_p, b11 = *e.b11_p;
-  extern __shared__ double sh[];
-  double *cr = sh, *ci = sh + r;                 // current LU row / work vector
-  double *br = sh + 2 * r, *bi = sh + 3 * r;     // right-hand side / solution
-  double *lr = sh + 4 * r, *li = sh + 5 * r;     // multipliers
-  int *swp = reinterpret_cast<int *>(sh + 6 * r);  // pivot swaps
-  double *red = sh + 6 * r + (r + 1) / 2 + 1;      // 32 doubles
-  double *zr_s = red + 32, *zi_s = zr_s + r;       // eigenvector z (r)
-  double *wr_s = zi_s + r, *wi_s = wr_s + r;       // left eigenvector w (r)
-  __shared__ cplx s_piv, s_l;
-  __shared__ int s_swap;
-  double *Ur = e.lu + size_t(blockIdx.x) * 2 * size_t(r) * r;  // U of the LU (r x r complex, col-major)
-  double *Ui = Ur + size_t(r) * r;
-  const double *Hs = e.Hs;
-  const int ldh = e.ld;
-  const double anorm = e.anorm[0];
-  const double tiny = 2.220446049250313e-16 * (anorm > 0.0 ? anorm : 1.0);
-  for (int idx = blockIdx.x; idx < r; idx += gridDim.x) {
-    const double lre = e.wr[idx], lim = e.wi[idx];
-    if (lim < 0.0) continue;  // filled by the +Im partner
-    const cplx lam = {lre, lim};
-    // ---- LU of A = Hs - lam I with adjacent-row pivoting
-    for (int c = threadIdx.x; c < r; c += blockDim.x) {
-      cr[c] = Hs[0 + int64_t(c) * ldh] - (c == 0 ? lam.re : 0.0);
-      ci[c] = (c == 0 ? -lam.im : 0.0);
-    }
-    __syncthreads();
-    for (int k = 0; k < r - 1; ++k) {
-      if (threadIdx.x == 0) {
-        const cplx cur = {cr[k], ci[k]};
-        const cplx nxt = {Hs[(k + 1) + int64_t(k) * ldh], 0.0};
-        const bool sw = cabs2(nxt) > cabs2(cur);
-        cplx piv = sw ? nxt : cur, oth = sw ? cur : nxt;
-        if (piv.re == 0.0 && piv.im == 0.0) piv.re = tiny;
-        s_swap = sw ? 1 : 0;
-        s_piv = piv;
-        s_l = cdiv(oth, piv);
-        swp[k] = s_swap;
-        lr[k] = s_l.re;
-        li[k] = s_l.im;
-      }
-      __syncthreads();
-      const int sw = s_swap;
-      const cplx l = s_l;
-      for (int c = k + threadIdx.x; c < r; c += blockDim.x) {
-        const cplx cur = {cr[c], ci[c]};
-        const cplx nxt = {Hs[(k + 1) + int64_t(c) * ldh] - (c == k + 1 ? lam.re : 0.0), (c == k + 1 ? -lam.im : 0.0)};
-        cplx piv = sw ? nxt : cur;
-        const cplx oth = sw ? cur : nxt;
-        if (c == k) piv = s_piv;
-        Ur[k + int64_t(c) * r] = piv.re;
-        Ui[k + int64_t(c) * r] = piv.im;
-        if (c > k) {
-          const cplx nw = csub(oth, cmul(l, piv));
-          cr[c] = nw.re;
-          ci[c] = nw.im;
-        }
-      }
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      cplx last = {cr[r - 1], ci[r - 1]};
-      if (last.re == 0.0 && last.im == 0.0) last.re = tiny;
-      Ur[(r - 1) + int64_t(r - 1) * r] = last.re;
-      Ui[(r - 1) + int64_t(r - 1) * r] = last.im;
-    }
-    __syncthreads();
-    // ---- two inverse-iteration solves each for A z = b (right) and A^H w = b (left)
-    for (int side = 0; side < 2; ++side) {
-      for (int c = threadIdx.x; c < r; c += blockDim.x) {
-        br[c] = 1.0;
-        bi[c] = 0.0;
-      }
-      __syncthreads();
-      for (int itn = 0; itn < 2; ++itn) {
-        if (side == 0) {
-          // forward elimination on b
-          if (threadIdx.x == 0) {
-            for (int k = 0; k < r - 1; ++k) {
-              if (swp[k]) {
-                double t = br[k]; br[k] = br[k + 1]; br[k + 1] = t;
-                t = bi[k]; bi[k] = bi[k + 1]; bi[k + 1] = t;
-              }
-              const cplx l = {lr[k], li[k]};
-              const cplx nb = csub({br[k + 1], bi[k + 1]}, cmul(l, {br[k], bi[k]}));
-              br[k + 1] = nb.re;
-              bi[k + 1] = nb.im;
-            }
-          }
-          __syncthreads();
-          // back substitution U z = b, column oriented
-          for (int i = r - 1; i >= 0; --i) {
-            if (threadIdx.x == 0) {
-              const cplx zi_ = cdiv({br[i], bi[i]}, {Ur[i + int64_t(i) * r], Ui[i + int64_t(i) * r]});
-              br[i] = zi_.re;
-              bi[i] = zi_.im;
-            }
-            __syncthreads();
-            const cplx zv = {br[i], bi[i]};
-            for (int k = threadIdx.x; k < i; k += blockDim.x) {
-              const cplx u = {Ur[k + int64_t(i) * r], Ui[k + int64_t(i) * r]};
-              const cplx nb = csub({br[k], bi[k]}, cmul(u, zv));
-              br[k] = nb.re;
-              bi[k] = nb.im;
-            }
-            __syncthreads();
-          }
-        } else {
-          // U^H y = b (forward), then apply E_k^H in reverse
-          for (int i = 0; i < r; ++i) {
-            if (threadIdx.x == 0) {
-              const cplx yv = cdiv({br[i], bi[i]}, cconj({Ur[i + int64_t(i) * r], Ui[i + int64_t(i) * r]}));
-              br[i] = yv.re;
-              bi[i] = yv.im;
-            }
-            __syncthreads();
-            const cplx yv = {br[i], bi[i]};
-            for (int k = i + 1 + threadIdx.x; k < r; k += blockDim.x) {
-              const cplx u = cconj({Ur[i + int64_t(k) * r], Ui[i + int64_t(k) * r]});
-              const cplx nb = csub({br[k], bi[k]}, cmul(u, yv));
-              br[k] = nb.re;
-              bi[k] = nb.im;
-            }
-            __syncthreads();
-          }
-          if (threadIdx.x == 0) {
-            for (int k = r - 2; k >= 0; --k) {
-              const cplx l = cconj({lr[k], li[k]});
-              const cplx nb = csub({br[k], bi[k]}, cmul(l, {br[k + 1], bi[k + 1]}));
-              br[k] = nb.re;
-              bi[k] = nb.im;
-              if (swp[k]) {
-                double t = br[k]; br[k] = br[k + 1]; br[k + 1] = t;
-                t = bi[k]; bi[k] = bi[k + 1]; bi[k + 1] = t;
-              }
-            }
-          }
-          __syncthreads();
-        }
-        // normalise
-        double s2 = 0.0;
-        for (int c = threadIdx.x; c < r; c += blockDim.x) s2 += br[c] * br[c] + bi[c] * bi[c];
-        s2 = block_sum(s2, red);
-        const double inv = s2 > 0.0 ? 1.0 / sqrt(s2) : 1.0;
-        for (int c = threadIdx.x; c < r; c += blockDim.x) {
-          br[c] *= inv;
-          bi[c] *= inv;
-        }
-        __syncthreads();
-      }
-      // map back to the coordinates of G: v = Q v_hs
-      double *dr = side == 0 ? zr_s : wr_s, *di = side == 0 ? zi_s : wi_s;
-      for (int i = threadIdx.x; i < r; i += blockDim.x) {
-        if (e.have_q) {
-          double sr = 0.0, si = 0.0;
-          for (int k = 0; k < r; ++k) {
-            const double q = e.Q[i + int64_t(k) * e.ld];
-            sr += q * br[k];
-            si += q * bi[k];
-          }
-          dr[i] = sr;
-          di[i] = si;
-        } else {
-          dr[i] = br[i];
-          di[i] = bi[i];
-        }
-      }
-      __syncthreads();
-    }
-    // ---- normalise z: unit norm, largest-magnitude entry real positive (lowest index on ties)
-    double s2 = 0.0;
-    for (int c = threadIdx.x; c < r; c += blockDim.x) s2 += zr_s[c] * zr_s[c] + zi_s[c] * zi_s[c];
-    s2 = block_sum(s2, red);
-    __shared__ int s_arg;
-    if (threadIdx.x == 0) {
-      double best = -1.0;
-      int arg = 0;
-      for (int c = 0; c < r; ++c) {
-        const double a2 = zr_s[c] * zr_s[c] + zi_s[c] * zi_s[c];
-        if (a2 > best * (1.0 + 1e-12)) {
-          best = a2;
-          arg = c;
-        }
-      }
-      s_arg = arg;
-    }
-    __syncthreads();
-    {
-      const cplx zk = {zr_s[s_arg], zi_s[s_arg]};
-      const double az = sqrt(cabs2(zk));
-      const double nrm = sqrt(s2);
-      const cplx ph = {zk.re / (az * nrm), -zk.im / (az * nrm)};  // conj(zk)/|zk| / |z|
-      __syncthreads();
-      for (int c = threadIdx.x; c < r; c += blockDim.x) {
-        const cplx v = cmul({zr_s[c], zi_s[c]}, ph);
-        zr_s[c] = v.re;
-        zi_s[c] = v.im;
-      }
-      __syncthreads();
-    }
-    // ---- amplitude c = (w^H b) / (w^H z), b = beta_11 U_r^T e_1
-    double n1r = 0.0, n1i = 0.0, d1r = 0.0, d1i = 0.0;
-    for (int c = threadIdx.x; c < r; c += blockDim.x) {
-      const double bc = b11 * (e.have_u ? e.U[0 + int64_t(c) * e.ld] : (c == 0 ? 1.0 : 0.0));
-      // conj(w) * b
-      n1r += wr_s[c] * bc;
-      n1i += -wi_s[c] * bc;
-      // conj(w) * z
-      d1r += wr_s[c] * zr_s[c] + wi_s[c] * zi_s[c];
-      d1i += wr_s[c] * zi_s[c] - wi_s[c] * zr_s[c];
-    }
-    n1r = block_sum(n1r, red);
-    n1i = block_sum(n1i, red);
-    d1r = block_sum(d1r, red);
-    d1i = block_sum(d1i, red);
-    const cplx amp = cdiv({n1r, n1i}, {d1r, d1i});
-    // ---- y = U_r z (m entries) into the output column idx
-    double *yr = e.yr + int64_t(idx) * e.ld, *yi = e.yi + int64_t(idx) * e.ld;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      if (e.have_u) {
-        double sr = 0.0, si = 0.0;
-        for (int k = 0; k < r; ++k) {
-          const double u = e.U[i + int64_t(k) * e.ld];
-          sr += u * zr_s[k];
-          si += u * zi_s[k];
-        }
-        yr[i] = sr;
-        yi[i] = si;
-      } else {
-        yr[i] = zr_s[i];
-        yi[i] = zi_s[i];
-      }
-    }
-    __syncthreads();
-    // ---- error indicator (Sec. 3.2.3)
-    double ind;
-    if (!e.have_u) {
-      const double zl2 = zr_s[m - 1] * zr_s[m - 1] + zi_s[m - 1] * zi_s[m - 1];
-      ind = fabs(hlast) * sqrt(zl2);
-    } else {
-      // t = H_m y; t <- t - U_r (U_r^T t); ind = sqrt(|t|^2 + |h y_m|^2)
-      double *tr = e.tw + size_t(blockIdx.x) * 2 * size_t(e.ld), *ti = tr + e.ld;
-      for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        double sr = 0.0, si = 0.0;
-        for (int k = (i > 0 ? i - 1 : 0); k < m; ++k) {
-          const double h = e.H[i + int64_t(k) * e.ldH];
-          sr += h * yr[k];
-          si += h * yi[k];
-        }
-        tr[i] = sr;
-        ti[i] = si;
-      }
-      __syncthreads();
-      // u = U_r^T t  (r entries, in br/bi)
-      for (int k = threadIdx.x; k < r; k += blockDim.x) {
-        double sr = 0.0, si = 0.0;
-        for (int i = 0; i < m; ++i) {
-          const double u = e.U[i + int64_t(k) * e.ld];
-          sr += u * tr[i];
-          si += u * ti[i];
-        }
-        br[k] = sr;
-        bi[k] = si;
-      }
-      __syncthreads();
-      double acc = 0.0;
-      for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        double sr = tr[i], si = ti[i];
-        for (int k = 0; k < r; ++k) {
-          const double u = e.U[i + int64_t(k) * e.ld];
-          sr -= u * br[k];
-          si -= u * bi[k];
-        }
-        acc += sr * sr + si * si;
-      }
-      acc = block_sum(acc, red);
-      const double hy2 = hlast * hlast * (yr[m - 1] * yr[m - 1] + yi[m - 1] * yi[m - 1]);
-      ind = sqrt(acc + hy2);
-    }
-    if (threadIdx.x == 0) {
-      e.amp_re[idx] = amp.re;
-      e.amp_im[idx] = amp.im;
-      e.ind[idx] = ind;
-      if (lim > 0.0 && idx + 1 < r) {
-        e.amp_re[idx + 1] = amp.re;
-        e.amp_im[idx + 1] = -amp.im;
-        e.ind[idx + 1] = ind;
-      }
-    }
-    if (lim > 0.0 && idx + 1 < r) {
-      double *yr2 = e.yr + int64_t(idx + 1) * e.ld, *yi2 = e.yi + int64_t(idx + 1) * e.ld;
-      for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        yr2[i] = yr[i];
-        yi2[i] = -yi[i];
-      }
-    }
-    __syncthreads();
-  }
-}
-
 // ------------------------------------------------------------------------------ ordering
 // key_i = |c_i| (a conjugate pair takes the larger of its two), order by key desc, |lambda| desc,
 // Im desc, index asc.  Writes the sorted eigenvalues, indicators, amplitudes and y columns.
@@ -1026,6 +690,8 @@ __global__ void order_kernel(EigArgs e, int nsel) {
   extern __shared__ double sh[];
   double *key = sh, *lab = sh + r;
   int *pos = reinterpret_cast<int *>(sh + 2 * r);
+  // |c| and |lambda| are not negative: their bits compare as integers (the FP64 pipe takes 64 cycles)
+  const long long *ki = reinterpret_cast<const long long *>(key), *li = reinterpret_cast<const long long *>(lab);
   for (int i = threadIdx.x; i < r; i += blockDim.x) {
     double k = hypot(e.amp_re[i], e.amp_im[i]);
     if (e.wi[i] > 0.0 && i + 1 < r) k = fmax(k, hypot(e.amp_re[i + 1], e.amp_im[i + 1]));
@@ -1038,8 +704,8 @@ __global__ void order_kernel(EigArgs e, int nsel) {
     int rank = 0;
     for (int k = 0; k < r; ++k) {
       bool before;
-      if (key[k] != key[i]) before = key[k] > key[i];
-      else if (lab[k] != lab[i]) before = lab[k] > lab[i];
+      if (ki[k] != ki[i]) before = ki[k] > ki[i];
+      else if (li[k] != li[i]) before = li[k] > li[i];
       else if (e.wi[k] != e.wi[i]) before = e.wi[k] > e.wi[i];
       else before = k < i;
       rank += before;
@@ -1064,19 +730,6 @@ __global__ void order_kernel(EigArgs e, int nsel) {
     e.ysr[i + int64_t(c) * e.ld] = e.yr[i + int64_t(src) * e.ld];
     e.ysi[i + int64_t(c) * e.ld] = e.yi[i + int64_t(src) * e.ld];
   }
-}
-
-// sum |Hs| over the Hessenberg band (for the pivot floor of inverse iteration)
-__global__ void anorm_kernel(const double *Hs, int ld, const int *isc, double *out) {
-  const int n = isc[ISC_R];
-  __shared__ double red[32];
-  double s = 0.0;
-  for (int64_t e = threadIdx.x; e < int64_t(n) * n; e += blockDim.x) {
-    const int i = int(e % n), c = int(e / n);
-    if (i <= c + 1) s += fabs(Hs[i + int64_t(c) * ld]);
-  }
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) out[0] = s;
 }
 
 }  // namespace foa

@@ -10,13 +10,13 @@
 
 namespace foa {
 
-static constexpr int kVecGridMax = 64;  // CTAs of the inverse-iteration kernel (each owns LU scratch)
+static constexpr int kVecGridMax = 304;  // CTAs of vectors_kernel (each owns 2 k_max doubles of scratch)
 static constexpr int kQrSmemMaxOrder = 160;  // largest order whose matrix (200 KB) the QR iteration keeps in shared memory
 
 static void free_work(EigWork *w) {
   void *ptrs[] = {w->A,  w->U,  w->sig_raw, w->sig, w->G,      w->Q,     w->T,     w->Aqr,   w->wr,
                   w->wi, w->yr, w->yi,      w->ysr, w->ysi,    w->ind,   w->amp_re, w->amp_im, w->out,
-                  w->anorm, w->lu, w->tw, w->yplanes, w->perm, w->isc, w->gb, w->bop, w->scal};
+                  w->rscal, w->vec, w->tw, w->yplanes, w->invsub, w->zr, w->zi, w->dold, w->conv, w->left, w->perm, w->isc, w->gb, w->bop, w->scal};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   delete w;
@@ -54,8 +54,10 @@ static int eig_alloc(foa_dmd *h, EigWork **slot) {
   } while (0)
   AL(w->A, K2); AL(w->U, K2); AL(w->sig_raw, K1); AL(w->sig, K1); AL(w->G, K2); AL(w->Q, K2); AL(w->T, K2);
   AL(w->Aqr, K2); AL(w->wr, K1); AL(w->wi, K1); AL(w->yr, K2); AL(w->yi, K2); AL(w->ysr, K2); AL(w->ysi, K2);
-  AL(w->ind, K1); AL(w->amp_re, K1); AL(w->amp_im, K1); AL(w->out, OUT_N * K1); AL(w->anorm, 8);
-  AL(w->lu, size_t(w->vgrid) * 2 * K2); AL(w->tw, size_t(w->vgrid) * 2 * K1); AL(w->yplanes, 2 * K2);
+  AL(w->ind, K1); AL(w->amp_re, K1); AL(w->amp_im, K1); AL(w->out, OUT_N * K1); AL(w->rscal, 4 * 8);
+  AL(w->vec, 4 * K2); AL(w->invsub, K1); AL(w->zr, 2 * K1); AL(w->zi, 2 * K1); AL(w->dold, K1);
+  AL(w->conv, size_t(K) * 4); AL(w->left, kRootSteps * 4);
+  AL(w->tw, size_t(w->vgrid) * 2 * K1); AL(w->yplanes, 2 * K2);
   AL(w->perm, size_t(K) * 4); AL(w->isc, ISC_N * 4); AL(w->gb, sizeof(GridBar));
   AL(w->bop, modes_tc_bop_bytes(K));
   AL(w->scal, 2 * 8);
@@ -130,10 +132,26 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
     }
     h->launches += 1;
   }
-  anorm_kernel<<<1, 512, 0, s>>>(w->G, K, w->isc, w->anorm);
+  RootArgs ra;
+  ra.H = w->G;
+  ra.invsub = w->invsub;
+  ra.zr = w->zr;
+  ra.zi = w->zi;
+  ra.dold = w->dold;
+  ra.conv = w->conv;
+  ra.left = w->left;
+  ra.scal = w->rscal;
+  ra.wr = w->wr;
+  ra.wi = w->wi;
+  ra.isc = w->isc;
+  ra.ld = K;
+  ra.min_n = kRootMinOrder;
+  e = launch_roots(ra, m, s);
+  if (e != cudaSuccess) return cuda_status(e);
   e = cudaMemcpyAsync(w->Aqr, w->G, size_t(K) * K * 8, cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return cuda_status(e);
-  // The QR iteration works on the r x r matrix (r = m without truncation); r is counted on the
+  // The QR iteration runs where the simultaneous iteration does not apply or has not converged
+  // (isc[ISC_QR]).  It works on the r x r matrix (r = m without truncation); r is counted on the
   // device.  The launch offers the band |j - i| <= 3 (7 m doubles) and up to 160^2 doubles for the
   // whole matrix, which the kernel copies to shared memory when r^2 fits (every truncated eig with
   // r <= 160, whatever m).
@@ -155,8 +173,9 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   a.ldH = K;
   a.wr = w->wr;
   a.wi = w->wi;
-  a.anorm = w->anorm;
-  a.lu = w->lu;
+  a.anorm = w->rscal;
+  a.M = w->T;  // the projection's scratch, free by now
+  a.vec = w->vec;
   a.tw = w->tw;
   a.yr = w->yr;
   a.yi = w->yi;
@@ -174,12 +193,12 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   a.have_u = trunc ? 1 : 0;
   a.hlast_p = trunc ? h->H + m + int64_t(m - 1) * K : w->scal;  // h_{m+1,m} (0 after a breakdown)
   a.b11_p = trunc ? h->B : w->scal + 1;
-  const int vgrid = m < w->vgrid ? m : w->vgrid;
-  const size_t vsmem = (size_t(m) * 10 + size_t(m + 1) / 2 + 64) * 8;
-  vectors_kernel<<<vgrid, 256, vsmem, s>>>(a);
+  e = launch_vectors(a, w->vgrid, s);
+  if (e != cudaSuccess) return cuda_status(e);
   if (nsel > m) nsel = m;
   order_kernel<<<1, 512, size_t(m) * 20 + 64, s>>>(a, nsel);
-  h->launches += 4;  // anorm, hqr, vectors, order
+  // roots_setup (steps, finish), hqr, flip, invit, vectors, order
+  h->launches += 6 + (m >= kRootMinOrder ? kRootSteps + 1 : 0);
   if (trunc && copied) {
     e = cudaEventRecord(copied, s);
     if (e != cudaSuccess) return cuda_status(e);

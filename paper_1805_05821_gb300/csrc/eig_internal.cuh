@@ -15,7 +15,7 @@ struct GridBar {
 };
 
 // integer scalars of one eigen-decomposition (device)
-enum { ISC_R = 0, ISC_STATUS = 1, ISC_ERR = 2, ISC_ROT = 3, ISC_SWEEPS = 4, ISC_N = 16 };
+enum { ISC_R = 0, ISC_STATUS = 1, ISC_ERR = 2, ISC_ROT = 3, ISC_SWEEPS = 4, ISC_QR = 5, ISC_ITS = 6, ISC_N = 16 };
 // rows of the sorted output block (each ld long)
 enum { OUT_LRE = 0, OUT_LIM = 1, OUT_IND = 2, OUT_ARE = 3, OUT_AIM = 4, OUT_N = 5 };
 
@@ -27,7 +27,9 @@ struct EigArgs {
   int ldH;
   const double *wr, *wi;
   const double *anorm;
-  double *lu, *tw;    // per-CTA scratch
+  double *M;          // Hs transposed and flipped about its antidiagonal (r x r, ld)
+  double *vec;        // inverse iteration: Re z, Im z, Re w, Im w planes of ld x ld (eigenvectors of Hs)
+  double *tw;         // per-CTA scratch
   double *yr, *yi;    // y_i = U_r z_i (m x r, ld), unsorted
   double *ysr, *ysi;  // sorted y columns
   double *ind, *amp_re, *amp_im;
@@ -39,6 +41,23 @@ struct EigArgs {
   const double *hlast_p;  // h_{m+1,m} (device)
   const double *b11_p;    // beta_{1,1} (device)
 };
+
+// Simultaneous iteration for the eigenvalues (eig_roots.cu)
+constexpr int kRootSteps = 36;   // steps at most; what has not converged by then goes to the QR iteration
+constexpr int kRootMinOrder = 16;  // below this order the QR iteration's few steps are as quick
+struct RootArgs {
+  const double *H;    // Hessenberg matrix (ld)
+  double *invsub;     // -1 / h_{i,i-1}
+  double *zr, *zi;    // 2 x ld: the values before and after a step
+  double *dold;       // size of each value's last correction
+  int *conv, *left;   // per value: converged; per step: values that had not
+  double *scal;       // see roots_setup_kernel
+  double *wr, *wi;
+  int *isc;
+  int ld, min_n;
+};
+cudaError_t launch_roots(const RootArgs &a, int m, cudaStream_t s);
+cudaError_t launch_vectors(const EigArgs &e, int vgrid, cudaStream_t s);
 
 // one push-time indicator (device ring written by the indicator stream)
 struct IndRecord {
@@ -52,11 +71,11 @@ struct EigWork {
   int vgrid = 0;
   double *A = nullptr, *U = nullptr, *sig_raw = nullptr, *sig = nullptr, *G = nullptr, *Q = nullptr, *T = nullptr,
          *Aqr = nullptr, *wr = nullptr, *wi = nullptr, *yr = nullptr, *yi = nullptr, *ysr = nullptr, *ysi = nullptr,
-         *ind = nullptr, *amp_re = nullptr, *amp_im = nullptr, *out = nullptr, *anorm = nullptr, *lu = nullptr,
-         *tw = nullptr, *yplanes = nullptr;
+         *ind = nullptr, *amp_re = nullptr, *amp_im = nullptr, *out = nullptr, *rscal = nullptr, *vec = nullptr,
+         *tw = nullptr, *yplanes = nullptr, *invsub = nullptr, *zr = nullptr, *zi = nullptr, *dold = nullptr;
   float *bop = nullptr;  // pre-split Y operand of the tensor-core mode product
   double *scal = nullptr;  // untruncated path: h_{m+1,m} and beta_11, copied with H_m
-  int *perm = nullptr, *isc = nullptr;
+  int *perm = nullptr, *isc = nullptr, *conv = nullptr, *left = nullptr;
   GridBar *gb = nullptr;
 };
 
@@ -76,9 +95,21 @@ __global__ void copy_h_kernel(const double *H, int ldh, int m, double *G, int ld
 __global__ void hessenberg_kernel(double *G, int ldg, double *Q, int ldq, const int *isc);
 __global__ void hqr_kernel(double *Ag, int lda, const int *isc_in, double *wr, double *wi, int *isc,
                            int smem_elems);
-__global__ void vectors_kernel(EigArgs e);
 __global__ void order_kernel(EigArgs e, int nsel);
-__global__ void anorm_kernel(const double *Hs, int ld, const int *isc, double *out);
+
+// sum over the CTA, in a fixed order; red: one double per warp
+__device__ __forceinline__ double block_sum(double v, double *red) {
+  v = warp_sum(v);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) red[w] = v;
+  __syncthreads();
+  double t = 0.0;
+  const int nw = blockDim.x >> 5;
+  for (int i = 0; i < nw; ++i) t += red[i];
+  __syncthreads();
+  return t;
+}
 
 size_t modes_tc_bop_bytes(int kmax);
 // modes.cu: Phi = V Y (Y: m x ncols real planes, ld), written to phi (ld_phi)
