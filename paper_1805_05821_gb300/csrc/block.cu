@@ -68,45 +68,7 @@ __global__ void __launch_bounds__(256) blockq1_kernel(BlockArgs a, foa_dmd_push_
     dot[tid] = t;
   }
   __syncthreads();
-  // deterministic cross-CTA reduction (groups of 8 CTAs, then groups)
-  const int len = P * P;
-  double *mypart = a.partials + size_t(blockIdx.x) * len;
-  if (tid < len) mypart[tid] = dot[tid];
-  __threadfence();
-  __syncthreads();
-  const int ngroups = (gridDim.x + kGroup - 1) / kGroup;
-  const int grp = blockIdx.x / kGroup;
-  const int gfirst = grp * kGroup;
-  const int gsize = min(kGroup, int(gridDim.x) - gfirst);
-  if (tid == 0) {
-    const unsigned t = atomicAdd(&a.gcount[grp], 1u);
-    sflag[2] = (t == unsigned(gsize - 1)) ? 1 : 0;
-  }
-  __syncthreads();
-  if (!sflag[2]) return;
-  __threadfence();
-  if (tid < len) {
-    double t = 0.0;
-    for (int b = 0; b < gsize; ++b) t += __ldcg(a.partials + size_t(gfirst + b) * len + tid);
-    a.gpart[size_t(grp) * len + tid] = t;
-  }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    a.gcount[grp] = 0u;
-    const unsigned t = atomicAdd(&bs->ticket[3], 1u);
-    sflag[2] = (t == unsigned(ngroups - 1)) ? 1 : 0;
-  }
-  __syncthreads();
-  if (!sflag[2]) return;
-  __threadfence();
-  if (tid < len) {
-    double t = 0.0;
-    for (int gq = 0; gq < ngroups; ++gq) t += __ldcg(a.gpart + size_t(gq) * len + tid);
-    dot[tid] = t;
-  }
-  if (tid == 0) bs->ticket[3] = 0u;
-  __syncthreads();
+  if (!grid_reduce<256>(a.partials, a.gpart, a.gcount, &bs->ticket[3], P * P, dot, P * P, sflag + 2, tid)) return;
   // ---------------- the last CTA
   const int j = a.j;
   const int K = a.kmax;

@@ -79,51 +79,6 @@ __device__ inline int chol_up(int p, const double *G, double *R) {
   return p;
 }
 
-// Cross-CTA reduction of len doubles over the T threads of each CTA (deterministic: CTA order
-// within groups of 8, then group order); returns true in the last CTA, with the sums in dot[0..len).
-template <int T>
-__device__ bool block_reduce(const BlockArgs &a, double *dot, int len, int mode, volatile int *sflag, int tid) {
-  double *mypart = a.partials + size_t(blockIdx.x) * len;
-  for (int c = tid; c < len; c += T) mypart[c] = dot[c];
-  __threadfence();
-  named_bar_sync(1, T);
-  const int ngroups = (gridDim.x + kGroup - 1) / kGroup;
-  const int grp = blockIdx.x / kGroup;
-  const int gfirst = grp * kGroup;
-  const int gsize = min(kGroup, int(gridDim.x) - gfirst);
-  if (tid == 0) {
-    const unsigned t = atomicAdd(&a.gcount[grp], 1u);
-    sflag[2] = (t == unsigned(gsize - 1)) ? 1 : 0;
-  }
-  named_bar_sync(1, T);
-  if (!sflag[2]) return false;
-  __threadfence();
-  double *gp = a.gpart + size_t(grp) * len;
-  for (int c = tid; c < len; c += T) {
-    double t = 0.0;
-    for (int b = 0; b < gsize; ++b) t += __ldcg(a.partials + size_t(gfirst + b) * len + c);
-    gp[c] = t;
-  }
-  __threadfence();
-  named_bar_sync(1, T);
-  if (tid == 0) {
-    a.gcount[grp] = 0u;
-    const unsigned t = atomicAdd(&a.bs->ticket[mode], 1u);
-    sflag[2] = (t == unsigned(ngroups - 1)) ? 1 : 0;
-  }
-  named_bar_sync(1, T);
-  if (!sflag[2]) return false;
-  __threadfence();
-  for (int c = tid; c < len; c += T) {
-    double t = 0.0;
-    for (int g = 0; g < ngroups; ++g) t += __ldcg(a.gpart + size_t(g) * len + c);
-    dot[c] = t;
-  }
-  if (tid == 0) a.bs->ticket[mode] = 0u;
-  named_bar_sync(1, T);
-  return true;
-}
-
 // Shape of a block pass at basis size j: T threads a CTA (256: two CTAs per SM, basis up to 256
 // columns; 512: one CTA per SM, up to 512) and fc columns per thread (a kernel instance: 2, 4, 6
 // or 8 for T = 256, 6 or 8 for T = 512; fc * P a multiple of 8).

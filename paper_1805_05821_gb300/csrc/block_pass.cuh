@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(T, 512 / T) block_pass_kernel(const BlockArgs 
     }
   }
   named_bar_sync(1, T);
-  if (!block_reduce<T>(a, dot, len, MODE, sflag, tid)) return;
+  if (!grid_reduce<T>(a.partials, a.gpart, a.gcount, &a.bs->ticket[MODE], len, dot, len, sflag + 2, tid)) return;
   // ---------------- the last CTA: the scalar part
   if constexpr (MODE == BLK_A) {
     for (int e = tid; e < j * P; e += T) a.C1[(e % P) * a.kmax + e / P] = dot[e];

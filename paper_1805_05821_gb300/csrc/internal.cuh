@@ -16,7 +16,7 @@ constexpr int kWarps = 8;          // consumer warps of a streaming-pass CTA
 constexpr int kConsumers = kWarps * 32;
 constexpr int kThreads = kConsumers + 32;  // + one producer warp that issues the bulk copies
 constexpr int kMaxK = 512;         // largest k_max
-constexpr int kGroup = 8;          // CTAs per first-level group of the cross-CTA reduction
+constexpr int kGroup = 16;         // CTAs per first-level group of the cross-CTA reduction (see grid_reduce)
 constexpr int kMaxR = 64;          // largest number of tiles in one pipeline stage
 constexpr int kMaxSlots = 8;
 
@@ -215,6 +215,80 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// Sum of one double per thread over the first kConsumers threads (v in nrm[tid], own slot), left in
+// *out: a shuffle tree per warp and one over the warps.  (One thread adding 256 values in turn takes
+// 256 x 64 cycles of GB300's FP64 pipe, 8 us in every pass: pass A at n = 16384, j <= 64 took 21.7 us
+// with it.)
+__device__ __forceinline__ void norm_reduce(double *nrm, double *out, int tid) {
+  const double v = warp_sum(nrm[tid]);
+  if ((tid & 31) == 0) nrm[tid] = v;
+  named_bar_sync(1, kConsumers);
+  if (tid < 32) {
+    double t = tid < kWarps ? nrm[32 * tid] : 0.0;
+#pragma unroll
+    for (int o = kWarps / 2; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (tid == 0) *out = t;
+  }
+}
+
+// p[0] + p[stride] + ... + p[(n-1) stride], read through L2, eight loads in flight
+__device__ __forceinline__ double sum_strided(const double *p, int n, size_t stride) {
+  double t0 = 0.0, t1 = 0.0;
+  for (int b = 0; b < n; b += 8) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = b + u < n ? __ldcg(p + size_t(b + u) * stride) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+      t0 += v[u];
+      t1 += v[u + 1];
+    }
+  }
+  return t0 + t1;
+}
+
+// Deterministic cross-CTA sum of dot[0..len) over the grid, by the T threads (threadIdx.x < T) of
+// each CTA: every CTA leaves its vector in `partials`, the last CTA of each group of kGroup (atomic
+// ticket) sums its group in CTA order, the last group sums the groups in group order.  Returns true in
+// that one CTA, with the sums in dot, after resetting the counters.  Both levels are chains of L2
+// round trips and 64-cycle FP64 additions, so the group size is near the square root of the 304 CTAs
+// of a full grid (16, then 19 terms; groups of 8 left 38 terms for the last CTA).
+template <int T>
+__device__ __forceinline__ bool grid_reduce(double *partials, double *gpart, uint32_t *gcount, uint32_t *ticket,
+                                            size_t stride, double *dot, int len, volatile int *flag, int tid) {
+  double *mypart = partials + size_t(blockIdx.x) * stride;
+  for (int c = tid; c < len; c += T) mypart[c] = dot[c];
+  __threadfence();
+  named_bar_sync(1, T);
+  const int ngroups = (gridDim.x + kGroup - 1) / kGroup;
+  const int grp = blockIdx.x / kGroup;
+  const int gfirst = grp * kGroup;
+  const int gsize = min(kGroup, int(gridDim.x) - gfirst);
+  if (tid == 0) {
+    const unsigned t = atomicAdd(&gcount[grp], 1u);
+    *flag = (t == unsigned(gsize - 1)) ? 1 : 0;
+  }
+  named_bar_sync(1, T);
+  if (!*flag) return false;
+  __threadfence();
+  double *gp = gpart + size_t(grp) * stride;
+  for (int c = tid; c < len; c += T) gp[c] = sum_strided(partials + size_t(gfirst) * stride + c, gsize, stride);
+  __threadfence();
+  named_bar_sync(1, T);
+  if (tid == 0) {
+    gcount[grp] = 0u;
+    const unsigned t = atomicAdd(ticket, 1u);
+    *flag = (t == unsigned(ngroups - 1)) ? 1 : 0;
+  }
+  named_bar_sync(1, T);
+  if (!*flag) return false;
+  __threadfence();
+  for (int c = tid; c < len; c += T) dot[c] = sum_strided(gpart + c, ngroups, stride);
+  if (tid == 0) *ticket = 0u;
+  named_bar_sync(1, T);
+  return true;
 }
 
 inline int dtype_size(int dt) { return dt == FOA_DMD_F64 ? 8 : dt == FOA_DMD_F32 ? 4 : 2; }

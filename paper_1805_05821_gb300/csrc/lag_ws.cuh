@@ -22,56 +22,16 @@ __device__ __forceinline__ void lag_epilogue(const PassArgs &a, DevState *st, do
                                              const double *pend_part, volatile int *sflag, const int j,
                                              const int jt, const int tid) {
   named_bar_sync(1, kConsumers);
-  if (tid == 0) {
-    double t = 0.0;
-    for (int i = 0; i < kConsumers; ++i) t += nrm[i];
-    dot[j] = t;
-    if (pend_part) {
-      double p = 0.0;
-      for (int w = 0; w < kWarps; ++w) p += pend_part[w];
-      dot[jt] = p;
-    }
+  norm_reduce(nrm, dot + j, tid);
+  if (tid == kConsumers - 1 && pend_part) {
+    double p = 0.0;
+    for (int w = 0; w < kWarps; ++w) p += pend_part[w];
+    dot[jt] = p;
   }
   named_bar_sync(1, kConsumers);
-  const int len = j + 1;
-  double *mypart = a.partials + size_t(blockIdx.x) * (a.kmax + 1);
-  for (int c = tid; c < len; c += kConsumers) mypart[c] = dot[c];
-  __threadfence();
-  named_bar_sync(1, kConsumers);
-  const int ngroups = (gridDim.x + kGroup - 1) / kGroup;
-  const int grp = blockIdx.x / kGroup;
-  const int gfirst = grp * kGroup;
-  const int gsize = min(kGroup, int(gridDim.x) - gfirst);
-  if (tid == 0) {
-    const unsigned t = atomicAdd(&a.gcount[grp], 1u);
-    sflag[2] = (t == unsigned(gsize - 1)) ? 1 : 0;
-  }
-  named_bar_sync(1, kConsumers);
-  if (!sflag[2]) return;
-  __threadfence();
-  double *gp = a.gpart + size_t(grp) * (a.kmax + 1);
-  for (int c = tid; c < len; c += kConsumers) {
-    double t = 0.0;
-    for (int bq = 0; bq < gsize; ++bq) t += __ldcg(a.partials + size_t(gfirst + bq) * (a.kmax + 1) + c);
-    gp[c] = t;
-  }
-  __threadfence();
-  named_bar_sync(1, kConsumers);
-  if (tid == 0) {
-    a.gcount[grp] = 0u;
-    const unsigned t = atomicAdd(&st->ticket[PASS_A2], 1u);
-    sflag[2] = (t == unsigned(ngroups - 1)) ? 1 : 0;
-  }
-  named_bar_sync(1, kConsumers);
-  if (!sflag[2]) return;
-  __threadfence();
-  for (int c = tid; c < len; c += kConsumers) {
-    double t = 0.0;
-    for (int g = 0; g < ngroups; ++g) t += __ldcg(a.gpart + size_t(g) * (a.kmax + 1) + c);
-    dot[c] = t;
-  }
-  if (tid == 0) st->ticket[PASS_A2] = 0u;
-  named_bar_sync(1, kConsumers);
+  if (!grid_reduce<kConsumers>(a.partials, a.gpart, a.gcount, &st->ticket[PASS_A2], a.kmax + 1, dot, j + 1, sflag + 2,
+                               tid))
+    return;
   for (int c = tid; c < j; c += kConsumers) a.hvec[c] = dot[c];
   if (tid == 0) {
     st->x_norm = sqrt(dot[j]);

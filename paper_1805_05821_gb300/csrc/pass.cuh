@@ -32,64 +32,22 @@ namespace foa {
 
 // Cross-CTA reduction and the scalar part of the step, shared by the streaming-pass kernels.
 // On entry every consumer thread (tid < kConsumers) has added its column partials into dot[0..j)
-// and stored its norm partial in nrm[tid]; dot[j] receives the CTA's norm.  Each CTA leaves its
-// FP64 partial vector in global memory; the last CTA of every group of 8 CTAs (atomic ticket)
-// sums its group in CTA order, and the last group sums the group partials in group order, so the
-// reduction is deterministic.  That last CTA then applies the scalar part of the step.
+// and stored its norm partial in nrm[tid]; dot[j] receives the CTA's norm (pass B has none).  The
+// last CTA of grid_reduce then applies the scalar part of the step.
 template <int MODE>
 __device__ __forceinline__ void pass_epilogue(const PassArgs &a, DevState *st, double *dot, double *nrm,
                                               volatile int *sflag, const int j, const int tid) {
   constexpr bool kNorm = (MODE == PASS_A || MODE == PASS_C || MODE == PASS_FIRST || MODE == PASS_B2);
   named_bar_sync(1, kConsumers);
-  const int len = j + 1;
-  if (tid == 0) {
-    if constexpr (kNorm) {
-      double t = 0.0;
-      for (int i = 0; i < kConsumers; ++i) t += nrm[i];
-      dot[j] = t;
-    }
+  if constexpr (kNorm) {
+    norm_reduce(nrm, dot + j, tid);
+    named_bar_sync(1, kConsumers);
   }
-  named_bar_sync(1, kConsumers);
-  double *mypart = a.partials + size_t(blockIdx.x) * (a.kmax + 1);
-  for (int c = tid; c < len; c += kConsumers) mypart[c] = dot[c];
-  __threadfence();
-  named_bar_sync(1, kConsumers);
-
-  // ---------------- two-level deterministic reduction (last arriving CTA of each group)
-  const int ngroups = (gridDim.x + kGroup - 1) / kGroup;
-  const int grp = blockIdx.x / kGroup;
-  const int gfirst = grp * kGroup;
-  const int gsize = min(kGroup, int(gridDim.x) - gfirst);
-  if (tid == 0) {
-    const unsigned t = atomicAdd(&a.gcount[grp], 1u);
-    sflag[2] = (t == unsigned(gsize - 1)) ? 1 : 0;
-  }
-  named_bar_sync(1, kConsumers);
-  if (!sflag[2]) return;
-  __threadfence();
-  double *gp = a.gpart + size_t(grp) * (a.kmax + 1);
-  for (int c = tid; c < len; c += kConsumers) {
-    double t = 0.0;
-    for (int b = 0; b < gsize; ++b) t += __ldcg(a.partials + size_t(gfirst + b) * (a.kmax + 1) + c);
-    gp[c] = t;
-  }
-  __threadfence();
-  named_bar_sync(1, kConsumers);
-  if (tid == 0) {
-    a.gcount[grp] = 0u;
-    const unsigned t = atomicAdd(&st->ticket[MODE], 1u);
-    sflag[2] = (t == unsigned(ngroups - 1)) ? 1 : 0;
-  }
-  named_bar_sync(1, kConsumers);
-  if (!sflag[2]) return;
-  __threadfence();
-  for (int c = tid; c < len; c += kConsumers) {
-    double t = 0.0;
-    for (int g = 0; g < ngroups; ++g) t += __ldcg(a.gpart + size_t(g) * (a.kmax + 1) + c);
-    dot[c] = t;
-  }
-  if (tid == 0) st->ticket[MODE] = 0u;
-  named_bar_sync(1, kConsumers);
+  // passes C and FIRST have no column dots: only the norm is summed
+  constexpr bool kNormOnly = (MODE == PASS_C || MODE == PASS_FIRST);
+  if (!grid_reduce<kConsumers>(a.partials, a.gpart, a.gcount, &st->ticket[MODE], a.kmax + 1, kNormOnly ? dot + j : dot,
+                               kNormOnly ? 1 : j + 1, sflag + 2, tid))
+    return;
 
   // ---------------- scalar part of the step (one CTA)
   if constexpr (MODE == PASS_A) {
@@ -192,11 +150,9 @@ __device__ __forceinline__ void pass_epilogue(const PassArgs &a, DevState *st, d
       t += sc * sc;
     }
     ssq[tid] = t;
-    named_bar_sync(1, kConsumers);
+    norm_reduce(ssq, ssq + 1, tid);
     if (tid == 0) {
-      double ss = 0.0;
-      for (int i = 0; i < kConsumers; ++i) ss += ssq[i];
-      const double d = dot[j] - ss;
+      const double d = dot[j] - ssq[1];
       ssq[0] = d > 0.0 ? sqrt(d) : 0.0;
     }
     named_bar_sync(1, kConsumers);
