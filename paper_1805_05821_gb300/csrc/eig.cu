@@ -1,9 +1,6 @@
 // Device eigen path of FOA-based DMD (the eigen extraction of Alg. 1 and Alg. 3), all in FP64:
 //
-//   svd_jacobi_kernel  one-sided (Hestenes) Jacobi SVD of the upper-triangular beta_m, run by a
-//                      cooperative grid: each round of the round-robin ordering rotates m/2
-//                      independent column pairs, one pair per CTA of four warps; beta_m W =
-//                      U Sigma gives U and Sigma without forming W (Sec. 3.2.2 rank truncation).
+//   eig_svd.cu         singular values and left singular vectors of beta_m (Sec. 3.2.2 rank truncation).
 //   project_t/g_kernel G = U_r^T H_m U_r (copy_h_kernel: G = H_m without truncation).
 //   hessenberg_kernel  Householder reduction of G to upper Hessenberg form G = Q Hs Q^T.
 //   eig_roots.cu       eigenvalues of Hs by simultaneous iteration, all SMs at work.
@@ -23,63 +20,6 @@
 
 namespace foa {
 
-// ------------------------------------------------------------------------------ grid barrier
-// Only used in cooperative launches (all CTAs co-resident).  Bounded spin: a CTA that has waited
-// spin_limit clock cycles for the others records FOA_DMD_ETIMEOUT and returns false, and its
-// caller returns at once, so a CTA that never arrives ends the whole grid within the limit.
-__device__ bool grid_barrier(GridBar *gb, int *err, long long spin_limit) {
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ok = 1;
-    volatile unsigned *vgen = &gb->gen;
-    const unsigned gen = *vgen;
-    __threadfence();
-    const unsigned arrived = atomicAdd(&gb->count, 1u);
-    if (arrived == gridDim.x - 1) {
-      gb->count = 0u;
-      __threadfence();
-      atomicAdd(&gb->gen, 1u);
-    } else {
-      const long long t0 = clock64();
-      while (*vgen == gen) {
-        if (clock64() - t0 > spin_limit) {
-          ok = 0;
-          atomicExch(err, FOA_DMD_ETIMEOUT);
-          break;
-        }
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return ok != 0;
-}
-
-// Bounded wait of CTA p for its neighbours p-1 and p+1 (those that exist among np CTAs) to have
-// finished `target` rounds of the Jacobi sweep; the columns they rotated are then visible.
-__device__ bool wait_neighbours(GridBar *gb, int p, int np, unsigned target, int *err, long long spin_limit) {
-  __shared__ int ok;
-  if (threadIdx.x == 0) {
-    ok = 1;
-    const long long t0 = clock64();
-    volatile unsigned *rd = gb->round;
-    for (int q = p - 1; q <= p + 1 && ok; q += 2) {
-      if (q < 0 || q >= np) continue;
-      while (rd[q] < target) {
-        if (clock64() - t0 > spin_limit) {
-          ok = 0;
-          atomicExch(err, FOA_DMD_ETIMEOUT);
-          break;
-        }
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return ok != 0;
-}
-
 __device__ __forceinline__ int block_max_int(int v, int *red) {
   for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -91,175 +31,6 @@ __device__ __forceinline__ int block_max_int(int v, int *red) {
   for (int i = 1; i < nw; ++i) t = max(t, red[i]);
   __syncthreads();
   return t;
-}
-
-// ------------------------------------------------------------------------------ SVD
-// One-sided Jacobi on the columns of A = beta_m (m x m, ld).  Rotating columns i, j with
-// alpha = |a_i|^2, beta = |a_j|^2, gamma = a_i.a_j:  zeta = (beta - alpha) / (2 gamma),
-// t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)), c = 1/sqrt(1+t^2), s = c t,
-// a_i <- c a_i - s a_j,  a_j <- s a_i + c a_j.  Converged when no pair has
-// |gamma| > tol sqrt(alpha beta).  Afterwards sigma_i = |a_i| and u_i = a_i / sigma_i.
-//
-// A CTA of four warps (one per SM sub-partition, so the pair's FP64 work uses all four FP64
-// pipes of the SM) takes one column pair at a time: each thread holds up to kSvdRows rows of both
-// columns in registers, the three dot products are summed in a fixed order (warp trees, then the
-// four warps), thread 0 forms the rotation, and every thread rotates its rows.  The grid has one
-// CTA per pair of the round-robin ordering ((m+1)/2 <= 256 CTAs).  In that ordering the two
-// columns pair p takes in round r+1 were held in round r by pairs p-1 and p+1 (checked for every
-// m <= 512), so between rounds a CTA waits only for its two neighbours' round counters, not for
-// the whole grid; one grid barrier per sweep sums the rotation counts for the convergence test.
-// Columns are read through L2 (__ldcg): a column that comes back to an SM it visited before must
-// not be served from that SM's L1.
-//
-// skip_cta (normally -1) and spin_limit serve foa_dmd_test_wait_fault: CTA skip_cta returns before
-// its first grid-barrier arrival, as a CTA that died would, and the others give up after
-// spin_limit cycles.
-__global__ void __launch_bounds__(kSvdThreads) svd_jacobi_kernel(const double *B, int ldb, int m, double *A, int lda,
-                                                                 double *sig, int *isc, GridBar *gb, int max_sweeps,
-                                                                 double tol, long long spin_limit, int skip_cta) {
-  int *err = isc + ISC_ERR;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t gtid = int64_t(blockIdx.x) * blockDim.x + tid;
-  const int64_t gthreads = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t e = gtid; e < int64_t(m) * m; e += gthreads) {
-    const int r = int(e % m), c = int(e / m);
-    A[r + int64_t(c) * lda] = (r <= c) ? B[r + int64_t(c) * ldb] : 0.0;
-  }
-  if (gtid == 0) isc[ISC_ROT] = 0;
-  if (int(blockIdx.x) == skip_cta) return;  // failure injection only (uniform over the CTA)
-  if (!grid_barrier(gb, err, spin_limit)) return;
-  __shared__ double red[kSvdThreads / 32][3];
-  __shared__ double rcs[2];
-  __shared__ int rgo, nrot;
-  const int mp = m + (m & 1);  // players of the round-robin schedule (m may be odd: one dummy)
-  const int npairs = mp / 2;
-  const double tol2 = tol * tol;
-  const bool nbr = int(gridDim.x) == npairs;  // one pair per CTA: neighbour waits between rounds
-  if (max_sweeps > kMaxSweeps) max_sweeps = kMaxSweeps;
-  unsigned gr = 0;  // rounds finished by this CTA
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    int myrot = 0;  // rotations applied by this CTA in the sweep (thread 0)
-    for (int rnd = 0; rnd < mp - 1; ++rnd) {
-      if (nbr && gr > 0 && !wait_neighbours(gb, blockIdx.x, npairs, gr, err, spin_limit)) return;
-      for (int p = blockIdx.x; p < npairs; p += gridDim.x) {
-        const int pa = p, pb = mp - 1 - p;
-        const int i = pa == 0 ? 0 : 1 + (pa - 1 + rnd) % (mp - 1);
-        const int j = pb == 0 ? 0 : 1 + (pb - 1 + rnd) % (mp - 1);
-        if (i >= m || j >= m) continue;  // uniform over the CTA
-        double *ai = A + int64_t(i) * lda, *aj = A + int64_t(j) * lda;
-        double x[kSvdRows], y[kSvdRows];
-        double al = 0.0, be = 0.0, ga = 0.0;
-#pragma unroll
-        for (int u = 0; u < kSvdRows; ++u) {
-          const int k = tid + u * kSvdThreads;
-          x[u] = k < m ? __ldcg(ai + k) : 0.0;
-          y[u] = k < m ? __ldcg(aj + k) : 0.0;
-          al = fma(x[u], x[u], al);
-          be = fma(y[u], y[u], be);
-          ga = fma(x[u], y[u], ga);
-        }
-        al = warp_sum(al);
-        be = warp_sum(be);
-        ga = warp_sum(ga);
-        if (lane == 0) {
-          red[warp][0] = al;
-          red[warp][1] = be;
-          red[warp][2] = ga;
-        }
-        __syncthreads();
-        if (tid == 0) {
-          double sa = 0.0, sb = 0.0, sg = 0.0;
-          for (int w = 0; w < kSvdThreads / 32; ++w) {
-            sa += red[w][0];
-            sb += red[w][1];
-            sg += red[w][2];
-          }
-          const int go = (sg != 0.0) && (sg * sg > tol2 * (sa * sb));
-          if (go) {
-            const double zeta = (sb - sa) / (2.0 * sg);
-            const double t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
-            const double c = rsqrt(fma(t, t, 1.0));
-            rcs[0] = c;
-            rcs[1] = c * t;
-            ++myrot;
-          }
-          rgo = go;
-        }
-        __syncthreads();
-        if (rgo) {
-          const double c = rcs[0], sn = rcs[1];
-#pragma unroll
-          for (int u = 0; u < kSvdRows; ++u) {
-            const int k = tid + u * kSvdThreads;
-            if (k < m) {
-              ai[k] = c * x[u] - sn * y[u];
-              aj[k] = sn * x[u] + c * y[u];
-            }
-          }
-        }
-      }
-      if (nbr) {
-        __syncthreads();  // this CTA's rotated columns are written
-        if (tid == 0) {
-          __threadfence();
-          atomicExch(&gb->round[blockIdx.x], gr + 1);
-        }
-      } else if (!grid_barrier(gb, err, spin_limit)) {
-        return;
-      }
-      ++gr;
-    }
-    if (tid == 0 && myrot) atomicAdd(&gb->rot[sweep], unsigned(myrot));
-    if (!grid_barrier(gb, err, spin_limit)) return;  // every CTA has finished the sweep and added its count
-    if (tid == 0) nrot = int(*(volatile unsigned *)&gb->rot[sweep]);
-    __syncthreads();
-    if (nrot == 0) break;
-  }
-  if (gtid == 0) isc[ISC_SWEEPS] = sweep;
-  // column norms (one warp per column)
-  const int warp_g = int(gtid >> 5), nwarps = int(gthreads >> 5);
-  for (int c = warp_g; c < m; c += nwarps) {
-    const double *ac = A + int64_t(c) * lda;
-    double sq = 0.0;
-    for (int k = lane; k < m; k += 32) {
-      const double v = __ldcg(ac + k);
-      sq += v * v;
-    }
-    sq = warp_sum(sq);
-    if (lane == 0) sig[c] = sqrt(sq);
-  }
-}
-
-// Sort singular values descending (stable by index), form U = A Sigma^{-1} in that order, and
-// count the retained rank r = #{sigma_i > tol sigma_1} (at least 1).  Single CTA.
-__global__ void svd_finish_kernel(const double *A, int lda, int m, const double *sig_in, double *U, double *sig,
-                                  int *isc, double rank_tol) {
-  extern __shared__ double sh[];
-  double *s = sh;                               // m
-  int *pos = reinterpret_cast<int *>(sh + m);   // m
-  for (int i = threadIdx.x; i < m; i += blockDim.x) s[i] = sig_in[i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    int rank = 0;
-    for (int k = 0; k < m; ++k) rank += (s[k] > s[i]) || (s[k] == s[i] && k < i);
-    pos[i] = rank;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < m; i += blockDim.x) sig[pos[i]] = s[i];
-  __syncthreads();
-  for (int64_t e = threadIdx.x; e < int64_t(m) * m; e += blockDim.x) {
-    const int r = int(e % m), c = int(e / m);
-    const double sc = s[c] > 0.0 ? 1.0 / s[c] : 0.0;
-    U[r + int64_t(pos[c]) * lda] = A[r + int64_t(c) * lda] * sc;
-  }
-  if (threadIdx.x == 0) {
-    double smax = 0.0;
-    for (int k = 0; k < m; ++k) smax = fmax(smax, s[k]);
-    int r = 0;
-    for (int k = 0; k < m; ++k) r += s[k] > rank_tol * smax;
-    isc[ISC_R] = r < 1 ? 1 : r;
-  }
 }
 
 // ------------------------------------------------------------------------------ projection

@@ -52,7 +52,7 @@ static int eig_alloc(foa_dmd *h, EigWork **slot) {
   do {                                                    \
     if (e == cudaSuccess) e = cudaMalloc((void **)&(p), (b)); \
   } while (0)
-  AL(w->A, K2); AL(w->U, K2); AL(w->sig_raw, K1); AL(w->sig, K1); AL(w->G, K2); AL(w->Q, K2); AL(w->T, K2);
+  AL(w->A, 2 * K2); AL(w->U, K2); AL(w->sig_raw, K1); AL(w->sig, K1); AL(w->G, K2); AL(w->Q, K2); AL(w->T, 2 * K2);
   AL(w->Aqr, K2); AL(w->wr, K1); AL(w->wi, K1); AL(w->yr, K2); AL(w->yi, K2); AL(w->ysr, K2); AL(w->ysi, K2);
   AL(w->ind, K1); AL(w->amp_re, K1); AL(w->amp_im, K1); AL(w->out, OUT_N * K1); AL(w->rscal, 4 * 8);
   AL(w->vec, 4 * K2); AL(w->invsub, K1); AL(w->zr, 2 * K1); AL(w->zi, 2 * K1); AL(w->dold, K1);
@@ -98,13 +98,13 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   else if (rank_tol < 0.0) tol = (m + 1) * eps_of(h->dtype);
   const bool trunc = tol > 0.0;
   if (trunc) {
-    // cooperative one-sided Jacobi SVD of beta_m (one CTA of four warps per column pair and round)
+    // cooperative one-sided Jacobi SVD of beta_m (one CTA per column pair and round)
     int grid = (m + 1) / 2;
     if (grid > 2 * h->sms) grid = 2 * h->sms;
     if (grid < 1) grid = 1;
     const double *Bp = h->B;
     int ldb = K, mm = m, lda = K, sweeps = 30, *iscp = w->isc;
-    double *Ap = w->A, *sigp = w->sig_raw, jt = 4.0 * std::ldexp(1.0, -53) * std::sqrt(double(m));
+    double *Ap = w->A, *Jp = w->T, *sigp = w->sig_raw, jt = 4.0 * std::ldexp(1.0, -53) * std::sqrt(double(m));
     GridBar *gbp = w->gb;
     long long spin = kGridSpinCycles;
     int skip = -1;
@@ -116,10 +116,10 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
     // a barrier that timed out keeps a partial count: every launch starts from a zeroed one
     e = cudaMemsetAsync(w->gb, 0, sizeof(GridBar), s);
     if (e != cudaSuccess) return cuda_status(e);
-    void *args[] = {&Bp, &ldb, &mm, &Ap, &lda, &sigp, &iscp, &gbp, &sweeps, &jt, &spin, &skip};
+    void *args[] = {&Bp, &ldb, &mm, &Ap, &Jp, &lda, &sigp, &iscp, &gbp, &sweeps, &jt, &spin, &skip};
     e = cudaLaunchCooperativeKernel((void *)svd_jacobi_kernel, grid, kSvdThreads, args, 0, s);
     if (e != cudaSuccess) return cuda_status(e);
-    svd_finish_kernel<<<1, 512, size_t(m) * 12 + 64, s>>>(w->A, K, m, w->sig_raw, w->U, w->sig, w->isc, tol);
+    svd_finish_kernel<<<m < 128 ? m : 128, 512, 0, s>>>(w->T, K, m, w->sig_raw, w->U, w->sig, w->isc, tol);
     project_t_kernel<<<h->sms * 2, 256, 0, s>>>(h->H, K, m, w->U, K, w->isc, w->T, K);
     project_g_kernel<<<h->sms * 2, 256, 0, s>>>(w->U, K, m, w->isc, w->T, K, w->G, K);
     hessenberg_kernel<<<1, 512, size_t(m) * 8 + 32 * 8, s>>>(w->G, K, w->Q, K, w->isc);

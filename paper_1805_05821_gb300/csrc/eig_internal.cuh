@@ -11,7 +11,6 @@ struct GridBar {
   unsigned count;                 // grid barrier: arrivals
   unsigned gen;                   // grid barrier: generation
   unsigned rot[kMaxSweeps];       // rotations applied in each sweep (summed over CTAs)
-  unsigned round[kMaxK / 2];      // rounds each CTA has finished (its neighbours wait on it)
 };
 
 // integer scalars of one eigen-decomposition (device)
@@ -79,12 +78,13 @@ struct EigWork {
   GridBar *gb = nullptr;
 };
 
-constexpr int kSvdThreads = 128;  // threads of a Jacobi SVD CTA (four warps per column pair)
-constexpr int kSvdRows = (kMaxK + kSvdThreads - 1) / kSvdThreads;
+constexpr int kSvdHalf = 128;           // threads that hold a column pair of A, and as many for J
+constexpr int kSvdThreads = 2 * kSvdHalf;
+constexpr int kSvdRows = (kMaxK + kSvdHalf - 1) / kSvdHalf;
 constexpr long long kGridSpinCycles = 1ll << 32;  // bounded wait of a grid barrier (about 2 s at 2 GHz)
-__global__ void svd_jacobi_kernel(const double *B, int ldb, int m, double *A, int lda, double *sig, int *isc,
+__global__ void svd_jacobi_kernel(const double *B, int ldb, int m, double *A, double *J, int lda, double *sig, int *isc,
                                   GridBar *gb, int max_sweeps, double tol, long long spin_limit, int skip_cta);
-__global__ void svd_finish_kernel(const double *A, int lda, int m, const double *sig_in, double *U, double *sig,
+__global__ void svd_finish_kernel(const double *J, int ld, int m, const double *sig_in, double *U, double *sig,
                                   int *isc, double rank_tol);
 __global__ void project_t_kernel(const double *H, int ldh, int m, const double *U, int ldu, const int *isc,
                                  double *T, int ldt);
