@@ -16,7 +16,7 @@ static constexpr int kQrSmemMaxOrder = 160;  // largest order whose matrix (200 
 static void free_work(EigWork *w) {
   void *ptrs[] = {w->A,  w->U,  w->sig_raw, w->sig, w->G,      w->Q,     w->T,     w->Aqr,   w->wr,
                   w->wi, w->yr, w->yi,      w->ysr, w->ysi,    w->ind,   w->amp_re, w->amp_im, w->out,
-                  w->rscal, w->vec, w->tw, w->yplanes, w->invsub, w->zr, w->zi, w->dold, w->conv, w->left, w->perm, w->isc, w->gb, w->bop, w->scal};
+                  w->rscal, w->vec, w->tw, w->yplanes, w->invsub, w->zr, w->zi, w->dold, w->conv, w->left, w->part, w->hf, w->perm, w->isc, w->gb, w->bop, w->scal};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   delete w;
@@ -54,9 +54,9 @@ static int eig_alloc(foa_dmd *h, EigWork **slot) {
   } while (0)
   AL(w->A, 2 * K2); AL(w->U, K2); AL(w->sig_raw, K1); AL(w->sig, K1); AL(w->G, K2); AL(w->Q, K2); AL(w->T, 2 * K2);
   AL(w->Aqr, K2); AL(w->wr, K1); AL(w->wi, K1); AL(w->yr, K2); AL(w->yi, K2); AL(w->ysr, K2); AL(w->ysi, K2);
-  AL(w->ind, K1); AL(w->amp_re, K1); AL(w->amp_im, K1); AL(w->out, OUT_N * K1); AL(w->rscal, 4 * 8);
+  AL(w->ind, K1); AL(w->amp_re, K1); AL(w->amp_im, K1); AL(w->out, OUT_N * K1); AL(w->rscal, 5 * 8);
   AL(w->vec, 4 * K2); AL(w->invsub, K1); AL(w->zr, 2 * K1); AL(w->zi, 2 * K1); AL(w->dold, K1);
-  AL(w->conv, size_t(K) * 4); AL(w->left, kRootSteps * 4);
+  AL(w->conv, size_t(K) * 4); AL(w->part, size_t(K) * 4); AL(w->hf, (size_t(K) + 1) * K * 4); AL(w->left, kRootSteps * 4);
   AL(w->tw, size_t(w->vgrid) * 2 * K1); AL(w->yplanes, 2 * K2);
   AL(w->perm, size_t(K) * 4); AL(w->isc, ISC_N * 4); AL(w->gb, sizeof(GridBar));
   AL(w->bop, modes_tc_bop_bytes(K));
@@ -135,6 +135,9 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   RootArgs ra;
   ra.H = w->G;
   ra.invsub = w->invsub;
+  ra.Hf = w->hf;
+  ra.invsubf = w->hf + size_t(K) * K;
+  ra.part = w->part;
   ra.zr = w->zr;
   ra.zi = w->zi;
   ra.dold = w->dold;
@@ -197,8 +200,8 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   if (e != cudaSuccess) return cuda_status(e);
   if (nsel > m) nsel = m;
   order_kernel<<<1, 512, size_t(m) * 20 + 64, s>>>(a, nsel);
-  // roots_setup (steps, finish), hqr, flip, invit, vectors, order
-  h->launches += 6 + (m >= kRootMinOrder ? kRootSteps + 1 : 0);
+  // roots_setup (start, steps, pair, finish), hqr, flip, invit, vectors, order
+  h->launches += 6 + (m >= kRootMinOrder ? kRootSteps32 + kRootSteps + 3 : 0);
   if (trunc && copied) {
     e = cudaEventRecord(copied, s);
     if (e != cudaSuccess) return cuda_status(e);

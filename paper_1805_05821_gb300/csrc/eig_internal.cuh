@@ -42,14 +42,17 @@ struct EigArgs {
 };
 
 // Simultaneous iteration for the eigenvalues (eig_roots.cu)
-constexpr int kRootSteps = 36;   // steps at most; what has not converged by then goes to the QR iteration
+constexpr int kRootSteps32 = 14; // steps in FP32
+constexpr int kRootSteps = 20;   // and in FP64, at most; what has not converged by then goes to the QR iteration
 constexpr int kRootMinOrder = 16;  // below this order the QR iteration's few steps are as quick
 struct RootArgs {
   const double *H;    // Hessenberg matrix (ld)
   double *invsub;     // -1 / h_{i,i-1}
+  float *Hf, *invsubf;  // the same rounded to FP32
   double *zr, *zi;    // 2 x ld: the values before and after a step
   double *dold;       // size of each value's last correction
-  int *conv, *left;   // per value: converged; per step: values that had not
+  int *conv, *left;   // per value: converged (1 in FP32, 2 in FP64); per FP64 step: values that had not
+  int *part;          // per value: the one nearest to its conjugate
   double *scal;       // see roots_setup_kernel
   double *wr, *wi;
   int *isc;
@@ -74,7 +77,8 @@ struct EigWork {
          *tw = nullptr, *yplanes = nullptr, *invsub = nullptr, *zr = nullptr, *zi = nullptr, *dold = nullptr;
   float *bop = nullptr;  // pre-split Y operand of the tensor-core mode product
   double *scal = nullptr;  // untruncated path: h_{m+1,m} and beta_11, copied with H_m
-  int *perm = nullptr, *isc = nullptr, *conv = nullptr, *left = nullptr;
+  int *perm = nullptr, *isc = nullptr, *conv = nullptr, *left = nullptr, *part = nullptr;
+  float *hf = nullptr;  // K x K, then K
   GridBar *gb = nullptr;
 };
 
@@ -96,6 +100,13 @@ __global__ void hessenberg_kernel(double *G, int ldg, double *Q, int ldq, const 
 __global__ void hqr_kernel(double *Ag, int lda, const int *isc_in, double *wr, double *wi, int *isc,
                            int smem_elems);
 __global__ void order_kernel(EigArgs e, int nsel);
+
+// v 2^(1023 - e) as a float (e a biased exponent, at least v's): -2 < result < 2, 0 below 2^-126
+__device__ __forceinline__ float scaled_float(double v, int e) {
+  const int hi = __double2hiint(v), ex = ((hi >> 20) & 0x7ff) - e + 127;
+  if (ex <= 0) return 0.f;
+  return __int_as_float((hi & 0x80000000) | (ex << 23) | ((hi & 0xfffff) << 3) | (unsigned(__double2loint(v)) >> 29));
+}
 
 // sum over the CTA, in a fixed order; red: one double per warp
 __device__ __forceinline__ double block_sum(double v, double *red) {

@@ -84,13 +84,6 @@ __device__ __forceinline__ bool load_pair(const double *a, const double *b, int 
   }
 }
 
-// v 2^(1023 - e) as a float (e a biased exponent, at least v's): -2 < result < 2, 0 below 2^-126
-__device__ __forceinline__ float scaled_float(double v, int e) {
-  const int hi = __double2hiint(v), ex = ((hi >> 20) & 0x7ff) - e + 127;
-  if (ex <= 0) return 0.f;
-  return __int_as_float((hi & 0x80000000) | (ex << 23) | ((hi & 0xfffff) << 3) | (unsigned(__double2loint(v)) >> 29));
-}
-
 __device__ __forceinline__ float sqrt_approx(float v) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
