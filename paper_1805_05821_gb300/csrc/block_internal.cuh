@@ -51,15 +51,6 @@ struct BlockArgs {
   double resolve;       // kBlockResolveUnits * u_s
 };
 
-// four consecutive rows of one column (16-byte aligned FP32, 8-byte aligned BF16) as floats
-__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ float4 ld4(const __nv_bfloat16 *p) {
-  const uint2 u = *reinterpret_cast<const uint2 *>(p);
-  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x));
-  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
-  return make_float4(a.x, a.y, b.x, b.y);
-}
-
 // upper Cholesky of the leading block of a P x P matrix (column-major, leading dimension kMaxP);
 // returns the columns factored (the first failing pivot, or p)
 __device__ inline int chol_up(int p, const double *G, double *R) {

@@ -184,6 +184,32 @@ __device__ __forceinline__ int named_bar_or(int id, int count, int pred) {
   return r;
 }
 
+// ------------------------------------------------------------------------------------------
+// Programmatic dependent launch.  The kernels of a push follow one another on one stream; each is
+// launched while its predecessor still runs (launch_pdl) and waits for it to complete (pdl_wait) before
+// it reads anything the predecessors write.  Every thread of every CTA passes pdl_wait, also where the
+// CTA has nothing to do: a kernel's completion then implies its predecessors'.  pdl_trigger, after
+// the wait, lets the next kernel start as CTAs of this one exit: its launch, barrier set-up and first V
+// tiles overlap this one's cross-CTA reduction.
+// ------------------------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(unsigned(grid));
+  c.blockDim = dim3(unsigned(block));
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
 // two adjacent rows of one column (8-byte or 4-byte aligned): FP32 values
 __device__ __forceinline__ float2 ld_pair(const float *p) { return *reinterpret_cast<const float2 *>(p); }
 __device__ __forceinline__ float2 ld_pair(const __nv_bfloat16 *p) {
@@ -191,6 +217,21 @@ __device__ __forceinline__ float2 ld_pair(const __nv_bfloat16 *p) {
 }
 __device__ __forceinline__ float2 ld_pair(const double *p) {
   return make_float2(float(p[0]), float(p[1]));  // not used on the FP64 path
+}
+
+// four adjacent rows of one column (16-byte or 8-byte aligned)
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16 *p) {
+  const uint2 u = *reinterpret_cast<const uint2 *>(p);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
+__device__ __forceinline__ void st4(__nv_bfloat16 *p, float4 v) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+  *reinterpret_cast<uint2 *>(p) =
+      make_uint2(*reinterpret_cast<const unsigned *>(&a), *reinterpret_cast<const unsigned *>(&b));
 }
 
 // storage -> compute conversions

@@ -14,8 +14,7 @@ static cudaError_t launch_lag_one(const PassArgs &a, int grid, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k<<<grid, kThreads, a.smem_total, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kThreads, a.smem_total, s, a);
 }
 
 template <typename S, int NC>
@@ -27,8 +26,7 @@ static cudaError_t launch_lag_ws_one(const PassArgs &a, int grid, cudaStream_t s
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k<<<grid, kThreads, a.smem_total, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kThreads, a.smem_total, s, a);
 }
 
 template <typename S, int FC>
@@ -40,8 +38,7 @@ static cudaError_t launch_lag_fused_one(const PassArgs &a, int grid, cudaStream_
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k<<<grid, kConsumers, a.smem_total, s>>>(a);  // no producer warp
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kConsumers, a.smem_total, s, a);  // no producer warp
 }
 
 template <typename S>

@@ -32,6 +32,8 @@ __global__ void __launch_bounds__(kThreads, lag_min_blocks<S, NC, FIN>()) lag_ke
   constexpr int kCombStride = kFp64 ? 256 : 512;  // entries of one row-combine vector
   extern __shared__ __align__(128) unsigned char smem[];
   DevState *st = a.st;
+  pdl_wait();
+  pdl_trigger();
   if (!FIN && !st->active) return;
   const int pend = st->pending;
   if (FIN && !pend) return;

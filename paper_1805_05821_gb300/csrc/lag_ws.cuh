@@ -44,6 +44,8 @@ __global__ void __launch_bounds__(kThreads, 2) lag_ws_kernel(const PassArgs a) {
   static_assert(sizeof(typename Compute<S>::T) == 4, "FP32/BF16 storage only");
   extern __shared__ __align__(128) unsigned char smem[];
   DevState *st = a.st;
+  pdl_wait();
+  pdl_trigger();
   if (!st->active) return;
   const int pend = st->pending;
   const int jp = st->pend_col;          // index of the pending column

@@ -225,6 +225,55 @@ __device__ __forceinline__ void pass_epilogue(const PassArgs &a, DevState *st, d
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// Filling the stage ring.  issue_v announces stage s (its V tiles and base slice) on the slot's barrier
+// and fetches the tiles; issue_base fetches the slice of x or w, when its producer has completed (a
+// partial x slice, for an unaligned x or the ragged end, is read from global memory instead).
+// ------------------------------------------------------------------------------------------
+template <typename BaseT, bool kBaseX>
+__device__ __forceinline__ uint32_t base_bytes(const PassArgs &a, int t0, int nt) {
+  const bool bulk = kBaseX ? (a.x_aligned && int64_t(t0 + nt) * kTile <= a.n) : true;
+  return bulk ? uint32_t(nt) * kTile * sizeof(BaseT) : 0u;
+}
+template <typename S, typename BaseT, bool kBaseX>
+__device__ __forceinline__ void issue_v(const PassArgs &a, int j, int slot, int s, unsigned char *slots, uint64_t *full) {
+  if (s >= a.nstages) return;
+  const int t0 = s * a.R, nt = min(a.R, a.ntiles - t0);
+  const uint32_t tile_bytes = uint32_t(kTile) * uint32_t(j) * sizeof(S);
+  unsigned char *dst = slots + size_t(slot) * a.slot_bytes;
+  mbar_arrive_expect_tx(&full[slot], uint32_t(nt) * tile_bytes + base_bytes<BaseT, kBaseX>(a, t0, nt));
+  if (tile_bytes && FOA_CHECK(t0 >= 0 && t0 + nt <= a.ntiles, kChkTile))
+    for (int k = 0; k < nt; ++k)
+      bulk_g2s(dst + size_t(k) * tile_bytes, static_cast<const S *>(a.V) + int64_t(t0 + k) * a.kmax * kTile, tile_bytes,
+               &full[slot]);
+}
+template <typename BaseT, bool kBaseX>
+__device__ __forceinline__ void issue_base(const PassArgs &a, const BaseT *bg, int slot, int s, unsigned char *slots,
+                                           uint64_t *full) {
+  if (s >= a.nstages) return;
+  const int t0 = s * a.R, nt = min(a.R, a.ntiles - t0);
+  const uint32_t bytes = base_bytes<BaseT, kBaseX>(a, t0, nt);
+  if (bytes) bulk_g2s(slots + size_t(slot) * a.slot_bytes + a.base_off, bg + int64_t(t0) * kTile, bytes, &full[slot]);
+}
+// Basis size whose V tiles may be fetched before the predecessor completes, 0 for none.  Passes B and C
+// follow a pass of the same push: its state is settled.  Pass A follows prep_kernel, which starts
+// the push with j = q; the last column of V and q were written before that kernel started.  (The two-pass push's second
+// pass reads a column its predecessor writes.)
+template <int MODE>
+__device__ __forceinline__ int prefetch_columns(const PassArgs &a, const DevState *st) {
+  if constexpr (MODE == PASS_A || MODE == PASS_B || MODE == PASS_C) {
+    const volatile DevState *v = st;
+    const int j = MODE == PASS_A ? v->q : (v->active ? v->j : 0);
+    return j >= 1 && j <= a.jcap ? j : 0;
+  }
+  return 0;
+}
+// Wait for the copies of the ring's first stages: a CTA must not exit with copies under way.
+__device__ __forceinline__ void drain(const PassArgs &a, uint64_t *full) {
+  for (int k = 0; k < a.slots; ++k)
+    if (blockIdx.x + k * gridDim.x < a.nstages) mbar_wait(&full[k], 0);
+}
+
 // Two CTAs per SM for the FP32/BF16 forms while the column accumulators fit (NC <= 48, i.e.
 // j <= 384): one CTA's barrier phases then overlap the other's compute.
 template <typename S, int NC>
@@ -243,11 +292,6 @@ __global__ void __launch_bounds__(kThreads, pass_min_blocks<S, NC>()) pass_kerne
 
   extern __shared__ __align__(128) unsigned char smem[];
   DevState *st = a.st;
-  if (!st->active) return;
-  const int j = (MODE == PASS_FIRST) ? 0 : st->j;
-  if (MODE != PASS_FIRST && (j < 1 || j > a.jcap)) return;
-  if (MODE == PASS_FIRST && st->j != 0) return;
-
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   unsigned char *slots = smem;
@@ -260,9 +304,6 @@ __global__ void __launch_bounds__(kThreads, pass_min_blocks<S, NC>()) pass_kerne
   uint64_t *empty = full + kMaxSlots;
   volatile int *sflag = reinterpret_cast<volatile int *>(empty + kMaxSlots);  // [0] abort [1] issued [2] last
 
-  // QR view (a.form): pass A projects x itself (w = x, no pre-vector)
-  const bool qr_a = (MODE == PASS_A) && a.form != 0;
-  const double cscale = (MODE == PASS_A && !qr_a) ? st->inv_bjj : 1.0;
   if (tid == 0) {
     for (int i = 0; i < a.slots; ++i) {
       mbar_init(&full[i], 1);
@@ -273,43 +314,45 @@ __global__ void __launch_bounds__(kThreads, pass_min_blocks<S, NC>()) pass_kerne
     sflag[2] = 0;
     mbar_fence_init();
   }
+  __syncthreads();
+  const BaseT *baseg = kBaseX ? static_cast<const BaseT *>(a.x) : static_cast<const BaseT *>(a.w);
+  constexpr int kIssuer = kWarps * 32;  // lane 0 of the producer warp
+  // the ring's first stages of V before the predecessor is waited for, their base slices after it
+  const int jp = prefetch_columns<MODE>(a, st);
+  if (tid == kIssuer && jp)
+    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, slots, full);
+  pdl_wait();
+  pdl_trigger();
+  if (tid == kIssuer && jp)
+    for (int k = 0; k < a.slots; ++k) issue_base<BaseT, kBaseX>(a, baseg, k, blockIdx.x + k * gridDim.x, slots, full);
+  const int j = (MODE == PASS_FIRST) ? 0 : st->j;
+  if (!st->active || (MODE == PASS_FIRST ? st->j != 0 : (j < 1 || j > a.jcap)) || (jp && jp != j)) {
+    if (tid == kIssuer && jp) drain(a, full);
+    return;
+  }
+  // QR view (a.form): pass A projects x itself (w = x, no pre-vector)
+  const bool qr_a = (MODE == PASS_A) && a.form != 0;
+  const double cscale = (MODE == PASS_A && !qr_a) ? st->inv_bjj : 1.0;
   for (int c = tid; c < ((j + 7) & ~3); c += kThreads) cf[c] = c < j ? static_cast<C>(a.coef[c]) : C(0);
   for (int c = tid; c <= j; c += kThreads) dot[c] = 0.0;
   __syncthreads();
 
-  const S *Vg = static_cast<const S *>(a.V);
-  const int64_t tile_elems = int64_t(a.kmax) * kTile;
-  const uint32_t tile_bytes = uint32_t(kTile) * uint32_t(j) * sizeof(S);
 
   if (warp == kWarps) {
     // ---------------------------------------------------------------- producer warp
     if (lane == 0) {
-      const BaseT *baseg = kBaseX ? static_cast<const BaseT *>(a.x) : static_cast<const BaseT *>(a.w);
       int it = 0;
       for (int s = blockIdx.x; s < a.nstages; s += gridDim.x, ++it) {
         const int slot = it % a.slots;
-        if (it >= a.slots) {
-          if (!mbar_wait(&empty[slot], ((it / a.slots) - 1) & 1)) {
-            sflag[0] = 1;
-            atomicExch(&st->err, FOA_DMD_ETIMEOUT);
-            break;
-          }
+        if (it < a.slots && jp) continue;  // under way
+        if (it >= a.slots && !mbar_wait(&empty[slot], ((it / a.slots) - 1) & 1)) {
+          sflag[0] = 1;
+          atomicExch(&st->err, FOA_DMD_ETIMEOUT);
+          break;
         }
         if (sflag[0]) break;
-        const int t0 = s * a.R;
-        const int nt = min(a.R, a.ntiles - t0);
-        const int64_t r0 = int64_t(t0) * kTile;
-        const bool base_bulk = kBaseX ? (a.x_aligned && r0 + int64_t(nt) * kTile <= a.n) : true;
-        const uint32_t bbytes = base_bulk ? uint32_t(nt) * kTile * sizeof(BaseT) : 0u;
-        unsigned char *dst = slots + size_t(slot) * a.slot_bytes;
-        mbar_arrive_expect_tx(&full[slot], uint32_t(nt) * tile_bytes + bbytes);
-        if (tile_bytes) {
-          if (FOA_CHECK(t0 >= 0 && t0 + nt <= a.ntiles, kChkTile))
-            for (int k = 0; k < nt; ++k)
-              bulk_g2s(dst + size_t(k) * tile_bytes, Vg + int64_t(t0 + k) * tile_elems, tile_bytes, &full[slot]);
-        }
-        if (bbytes) bulk_g2s(dst + a.base_off, baseg + r0, bbytes, &full[slot]);
-        sflag[1] = it + 1;
+        issue_v<S, BaseT, kBaseX>(a, j, slot, s, slots, full);
+        issue_base<BaseT, kBaseX>(a, baseg, slot, s, slots, full);
       }
     }
     return;

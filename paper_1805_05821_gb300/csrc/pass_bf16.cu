@@ -14,8 +14,7 @@ static cudaError_t launch_one(const PassArgs &a, int grid, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k<<<grid, kThreads, a.smem_total, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kThreads, a.smem_total, s, a);
 }
 
 // passes with column dots: the warp-specialised kernel
@@ -28,8 +27,7 @@ static cudaError_t launch_ws_one(const PassArgs &a, int grid, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k<<<grid, kThreads, a.smem_total, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kThreads, a.smem_total, s, a);
 }
 
 // wide-basis stages (one or two tiles) held in registers: pass_fused_kernel
@@ -42,8 +40,7 @@ static cudaError_t launch_fused_one(const PassArgs &a, int grid, cudaStream_t s)
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k<<<grid, kConsumers, a.smem_total, s>>>(a);  // no producer warp
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kConsumers, a.smem_total, s, a);  // no producer warp
 }
 
 // passes with column dots (A, B, B2): the register-held kernel where its column groups fit,

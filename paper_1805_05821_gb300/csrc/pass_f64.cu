@@ -12,8 +12,7 @@ static cudaError_t launch_one(const PassArgs &a, int grid, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k<<<grid, kThreads, a.smem_total, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kThreads, a.smem_total, s, a);
 }
 
 template <int MODE>

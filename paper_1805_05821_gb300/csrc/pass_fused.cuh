@@ -38,10 +38,6 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
 
   extern __shared__ __align__(128) unsigned char smem[];
   DevState *st = a.st;
-  if (!st->active) return;
-  const int j = st->j;
-  if (j < 1 || j > a.jcap) return;
-
   const int tid = threadIdx.x;
   unsigned char *slots = smem;
   float *ws = reinterpret_cast<float *>(smem + a.off_ws);      // w of the stage's rows
@@ -52,14 +48,32 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + a.off_bar);
   volatile int *sflag = reinterpret_cast<volatile int *>(full + 2 * kMaxSlots);  // [0] abort [2] last
 
-  const bool qr_a = (MODE == PASS_A) && a.form != 0;
-  const float cscale = (MODE == PASS_A && !qr_a) ? float(st->inv_bjj) : 1.f;
   if (tid == 0) {
     for (int i = 0; i < a.slots; ++i) mbar_init(&full[i], 1);
     sflag[0] = 0;
     sflag[2] = 0;
     mbar_fence_init();
   }
+  __syncthreads();
+  // one elected thread issues the copies of a stage: R whole tiles of V and the stage's slice of x
+  // (pass A) or w; a partial x slice (unaligned x, ragged end) is read from global memory instead
+  const BaseT *bg = kBaseX ? static_cast<const BaseT *>(a.x) : static_cast<const BaseT *>(a.w);
+  constexpr int kIssuer = kConsumers - 1;  // not one of the row finishers (tid < 64)
+  // the ring's first stages of V before the predecessor is waited for, their base slices after it
+  const int jp = prefetch_columns<MODE>(a, st);
+  if (tid == kIssuer && jp)
+    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, slots, full);
+  pdl_wait();
+  pdl_trigger();
+  if (tid == kIssuer && jp)
+    for (int k = 0; k < a.slots; ++k) issue_base<BaseT, kBaseX>(a, bg, k, blockIdx.x + k * gridDim.x, slots, full);
+  const int j = st->j;
+  if (!st->active || j < 1 || j > a.jcap || (jp && jp != j)) {
+    if (tid == kIssuer && jp) drain(a, full);
+    return;
+  }
+  const bool qr_a = (MODE == PASS_A) && a.form != 0;
+  const float cscale = (MODE == PASS_A && !qr_a) ? float(st->inv_bjj) : 1.f;
   // fixed mapping: PF row pairs per full stage (R tiles), G1 column groups of cpg columns
   const int PF = a.R * (kTile / 2);                   // 16 (R = 1) or 32 (R = 2)
   const int G1 = kConsumers / PF;                     // 16 or 8
@@ -69,33 +83,12 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
   for (int c = tid; c <= j; c += kConsumers) dot[c] = 0.0;
   __syncthreads();
 
-  const S *Vg = static_cast<const S *>(a.V);
-  const int64_t tile_elems = int64_t(a.kmax) * kTile;
-  const uint32_t tile_bytes = uint32_t(kTile) * uint32_t(j) * sizeof(S);
-
-  // one elected thread issues the copies of a stage: R whole tiles of V and the stage's slice of x
-  // (pass A) or w; a partial x slice (unaligned x, ragged end) is read from global memory instead
-  const BaseT *bg = kBaseX ? static_cast<const BaseT *>(a.x) : static_cast<const BaseT *>(a.w);
-  constexpr int kIssuer = kConsumers - 1;  // not one of the row finishers (tid < 64)
   auto issue = [&](int slot, int s) {
-    const int t0 = s * a.R;
-    const int nt = min(a.R, a.ntiles - t0);
-    const int64_t r0 = int64_t(t0) * kTile;
-    const bool base_bulk = kBaseX ? (a.x_aligned && r0 + int64_t(nt) * kTile <= a.n) : true;
-    const uint32_t bbytes = base_bulk ? uint32_t(nt) * kTile * sizeof(BaseT) : 0u;
-    unsigned char *dst = slots + size_t(slot) * a.slot_bytes;
-    mbar_arrive_expect_tx(&full[slot], uint32_t(nt) * tile_bytes + bbytes);
-    if (FOA_CHECK(t0 >= 0 && t0 + nt <= a.ntiles, kChkTile))
-      for (int k = 0; k < nt; ++k)
-        bulk_g2s(dst + size_t(k) * tile_bytes, Vg + int64_t(t0 + k) * tile_elems, tile_bytes, &full[slot]);
-    if (bbytes) bulk_g2s(dst + a.base_off, bg + r0, bbytes, &full[slot]);
+    issue_v<S, BaseT, kBaseX>(a, j, slot, s, slots, full);
+    issue_base<BaseT, kBaseX>(a, bg, slot, s, slots, full);
   };
-  if (tid == kIssuer)
-    for (int k = 0; k < a.slots; ++k) {
-      const int s = blockIdx.x + k * gridDim.x;
-      if (s >= a.nstages) break;
-      issue(k, s);
-    }
+  if (tid == kIssuer && !jp)
+    for (int k = 0; k < a.slots; ++k) issue(k, blockIdx.x + k * gridDim.x);
 
   // ------------------------------------------------------------------ compute
   const int g = tid / PF, pr = tid % PF;
@@ -168,8 +161,7 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
     }
     named_bar_sync(1, kConsumers);  // every thread holds its fragment: the slot is free
     if (tid == kIssuer && !sflag[0]) {
-      const int sn = s + a.slots * gridDim.x;
-      if (sn < a.nstages) issue(slot, sn);
+      issue(slot, s + a.slots * gridDim.x);
     }
     if (tid < RS) {
       float acc = 0.f;

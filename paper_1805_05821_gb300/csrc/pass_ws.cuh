@@ -30,10 +30,6 @@ __global__ void __launch_bounds__(kThreads, 2) pass_ws_kernel(const PassArgs a) 
 
   extern __shared__ __align__(128) unsigned char smem[];
   DevState *st = a.st;
-  if (!st->active) return;
-  const int j = st->j;
-  if (j < 1 || j > a.jcap) return;
-
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   unsigned char *slots = smem;
@@ -48,9 +44,6 @@ __global__ void __launch_bounds__(kThreads, 2) pass_ws_kernel(const PassArgs a) 
   uint64_t *ws_full = empty + kMaxSlots + 2;
   uint64_t *ws_empty = ws_full + 2;
 
-  // QR view (a.form): pass A projects x itself (w = x, no pre-vector)
-  const bool qr_a = (MODE == PASS_A) && a.form != 0;
-  const float cscale = (MODE == PASS_A && !qr_a) ? float(st->inv_bjj) : 1.f;
   if (tid == 0) {
     for (int i = 0; i < a.slots; ++i) {
       mbar_init(&full[i], 1);
@@ -64,38 +57,45 @@ __global__ void __launch_bounds__(kThreads, 2) pass_ws_kernel(const PassArgs a) 
     sflag[2] = 0;
     mbar_fence_init();
   }
+  __syncthreads();
+  const BaseT *baseg = kBaseX ? static_cast<const BaseT *>(a.x) : static_cast<const BaseT *>(a.w);
+  constexpr int kIssuer = kWarps * 32;  // lane 0 of the producer warp
+  // the ring's first stages of V before the predecessor is waited for, their base slices after it
+  const int jp = prefetch_columns<MODE>(a, st);
+  if (tid == kIssuer && jp)
+    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, slots, full);
+  pdl_wait();
+  pdl_trigger();
+  if (tid == kIssuer && jp)
+    for (int k = 0; k < a.slots; ++k) issue_base<BaseT, kBaseX>(a, baseg, k, blockIdx.x + k * gridDim.x, slots, full);
+  const int j = st->j;
+  if (!st->active || j < 1 || j > a.jcap || (jp && jp != j)) {
+    if (tid == kIssuer && jp) drain(a, full);
+    return;
+  }
+  // QR view (a.form): pass A projects x itself (w = x, no pre-vector)
+  const bool qr_a = (MODE == PASS_A) && a.form != 0;
+  const float cscale = (MODE == PASS_A && !qr_a) ? float(st->inv_bjj) : 1.f;
   for (int c = tid; c < ((j + 7) & ~3); c += kThreads) cf[c] = c < j ? static_cast<float>(a.coef[c]) : 0.f;
   for (int c = tid; c <= j; c += kThreads) dot[c] = 0.0;
   __syncthreads();
 
-  const S *Vg = static_cast<const S *>(a.V);
-  const int64_t tile_elems = int64_t(a.kmax) * kTile;
-  const uint32_t tile_bytes = uint32_t(kTile) * uint32_t(j) * sizeof(S);
 
   if (warp == kWarps) {
     // ---------------------------------------------------------------- producer warp
     if (lane == 0) {
-      const BaseT *baseg = kBaseX ? static_cast<const BaseT *>(a.x) : static_cast<const BaseT *>(a.w);
       int it = 0;
       for (int s = blockIdx.x; s < a.nstages; s += gridDim.x, ++it) {
         const int slot = it % a.slots;
+        if (it < a.slots && jp) continue;  // under way
         if (it >= a.slots && !mbar_wait(&empty[slot], ((it / a.slots) - 1) & 1)) {
           sflag[0] = 1;
           atomicExch(&st->err, FOA_DMD_ETIMEOUT);
           break;
         }
         if (sflag[0]) break;
-        const int t0 = s * a.R;
-        const int nt = min(a.R, a.ntiles - t0);
-        const int64_t r0 = int64_t(t0) * kTile;
-        const bool base_bulk = kBaseX ? (a.x_aligned && r0 + int64_t(nt) * kTile <= a.n) : true;
-        const uint32_t bbytes = base_bulk ? uint32_t(nt) * kTile * sizeof(BaseT) : 0u;
-        unsigned char *dst = slots + size_t(slot) * a.slot_bytes;
-        mbar_arrive_expect_tx(&full[slot], uint32_t(nt) * tile_bytes + bbytes);
-        if (FOA_CHECK(t0 >= 0 && t0 + nt <= a.ntiles, kChkTile))
-          for (int k = 0; k < nt; ++k)
-            bulk_g2s(dst + size_t(k) * tile_bytes, Vg + int64_t(t0 + k) * tile_elems, tile_bytes, &full[slot]);
-        if (bbytes) bulk_g2s(dst + a.base_off, baseg + r0, bbytes, &full[slot]);
+        issue_v<S, BaseT, kBaseX>(a, j, slot, s, slots, full);
+        issue_base<BaseT, kBaseX>(a, baseg, slot, s, slots, full);
       }
     }
     return;
