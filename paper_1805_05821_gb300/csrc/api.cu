@@ -38,6 +38,12 @@ bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n,
   } else {
     while (R * 2 <= kMaxR && (R * 2) * tile_bytes <= g.stage_bytes) R *= 2;
   }
+  // FP64 storage is bound by the FP64 pipes (2 FMAs a clock and SM): few tiles are spread over all SMs in
+  // smaller stages, down to 8 KB.  (n = 4096, 11 pushes and the solve: 1.67 -> 1.30 ms.  FP32 stages
+  // stay: a pass of 32 KB a CTA is bound by its launch and reduction, which more CTAs make longer, 12
+  // against 17 us at n = 16384.)
+  if (cs == 8)
+    while (R > 1 && R * tile_bytes > 8192 && (ntiles + R - 1) / R < 4 * sms) R /= 2;
   const int64_t vpart = align_up(R * tile_bytes, 128);
   // the lagged first pass also stages the x slice (storage type) and the w' slice (compute type)
   const int64_t bpart = lag ? align_up(int64_t(R) * kTile * s, 128) + align_up(int64_t(R) * kTile * cs, 128)
