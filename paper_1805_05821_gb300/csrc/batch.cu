@@ -4,7 +4,7 @@
 //
 //   plan_kernel     reads every stream's device state and the caller's pointer array, decides
 //                   which streams push, and cuts each stream's passes into work items of whole
-//                   pipeline stages (about 8 MB of V each);
+//                   pipeline stages (128 KB to 8 MB of V, about six items a CTA);
 //   prep_kernel     beta_pre of every active stream (Alg. 1), one CTA per stream;
 //   bpass_kernel    pass A, then pass B, then pass C (pre-vector, CGS2, norm; Alg. 1) of all streams, one
 //                   launch per pass: two CTAs of 256 threads per SM take items from a counter;
@@ -40,8 +40,14 @@ constexpr int kStageCols = 256;             // R * j <= this while R > 1: stages
 constexpr int kRingBytes = 102400;          // the stage ring of a CTA (two 50 KB slots hold j <= 399)
 constexpr int kMaxBSlots = 6;
 constexpr int kCf = 640;                    // padded coefficient vector (>= 16 * 32 + 32)
-constexpr int64_t kItemBytes = 8ll << 20;   // V bytes per work item ...
-constexpr int kItemStages = 256;            // ... and at most this many stages
+// V bytes per work item.  The CTAs take items from a counter, so a pass ends unevenly by up to one item
+// a CTA, while every item fills the ring anew and writes its partial sums (about 4 us): six items a CTA,
+// within these limits.  With 8 MB throughout, a round of 48 streams (16k to 1M values, 1.9 GB of V)
+// was 240 items for 304 CTAs: 438 us a pass, now 363 us.
+constexpr int64_t kItemBytesMax = 8ll << 20, kItemBytesMin = 128ll << 10;
+constexpr int kItemsPerCta = 6;
+constexpr int kItemStages = 256;            // at most this many stages ...
+constexpr int kStreamItems = 512;           // ... and this many items of one stream (summed by one CTA)
 enum { PH_A = 0, PH_B = 1, PH_C = 2, PH_APP = 3, NPH = 4 };
 
 // shared-memory layout of bpass_kernel (bytes); two CTAs share an SM's 228 KB
@@ -61,11 +67,8 @@ struct StreamDesc {
   int64_t w_off;    // element offset of w
   int64_t mat_off;  // double offset of its k_max x k_max H-bar and beta
   int64_t vec_off;  // double offset of its pre/h/s vectors (3 x k_max)
-  int64_t part_off; // double offset of its item partials
   int32_t ntiles;
   int32_t kmax;
-  int32_t max_chunks;
-  int32_t pad;
 };
 
 struct BState {
@@ -89,7 +92,9 @@ struct BatchArgs {
   float *W;            // pool of w vectors (FP32)
   double *H, *B;       // pools
   double *vec;         // pools of pre/h/s
-  double *part;        // item partials
+  double *part;        // partials of a pass's items, by item
+  int32_t pstride;     // doubles of one item's partials
+  int32_t ctas;        // CTAs of a pass
   const void *const *x;  // caller's pointers (device array of S)
   double *h_last;      // caller's output array (device, S)
   double tol;
@@ -105,9 +110,27 @@ __host__ __device__ __forceinline__ int stage_tiles(int j) {
   return R;
 }
 
+// stages of one item for `goal` bytes
+__host__ __device__ __forceinline__ int item_stages(int64_t goal, int64_t stage_bytes) {
+  const int64_t cs = goal / stage_bytes;
+  return cs > kItemStages ? kItemStages : cs < 1 ? 1 : int(cs);
+}
+
 __global__ void plan_kernel(BatchArgs a, int ssize) {
   const int S = a.S;
   extern __shared__ int32_t cnt[];  // NPH * S counts
+  __shared__ unsigned long long bytes;
+  if (threadIdx.x == 0) bytes = 0ull;
+  __syncthreads();
+  for (int s = threadIdx.x; s < S; s += blockDim.x) {  // V bytes of this round
+    const BState &b = a.st[s];
+    const StreamDesc d = a.sd[s];
+    if (a.x[s] && !b.stopped && b.q < d.kmax)
+      atomicAdd(&bytes, (unsigned long long)(int64_t(d.ntiles) * kTile * max(b.q, 1) * ssize));
+  }
+  __syncthreads();
+  int64_t goal = int64_t(bytes) / (int64_t(a.ctas) * kItemsPerCta);
+  goal = goal < kItemBytesMin ? kItemBytesMin : goal > kItemBytesMax ? kItemBytesMax : goal;
   for (int s = threadIdx.x; s < S; s += blockDim.x) {
     const StreamDesc d = a.sd[s];
     BState &b = a.st[s];
@@ -125,14 +148,9 @@ __global__ void plan_kernel(BatchArgs a, int ssize) {
     p.R = stage_tiles(j);
     p.nstages = (d.ntiles + p.R - 1) / p.R;
     const int64_t stage_bytes = int64_t(p.R) * kTile * (j > 0 ? j : 1) * ssize;
-    p.cs = int(kItemBytes / stage_bytes);
-    if (p.cs > kItemStages) p.cs = kItemStages;
-    if (p.cs < 1) p.cs = 1;
+    p.cs = item_stages(goal, stage_bytes);
+    p.cs = max(p.cs, (p.nstages + kStreamItems - 1) / kStreamItems);
     p.nchunks = (p.nstages + p.cs - 1) / p.cs;
-    if (p.nchunks > d.max_chunks) {  // keep within the partials buffer
-      p.cs = (p.nstages + d.max_chunks - 1) / d.max_chunks;
-      p.nchunks = (p.nstages + p.cs - 1) / p.cs;
-    }
     a.plan[s] = p;
     const bool first = (j == 0);
     cnt[PH_A * S + s] = active ? p.nchunks : 0;               // pass A (or the first snapshot's norm)
@@ -444,8 +462,9 @@ __global__ void __launch_bounds__(kBT, 2) bpass_kernel(BatchArgs a, int ph) {
       dot[j] = t;
     }
     __syncthreads();
-    double *pp = a.part + sd.part_off + int64_t(chunk) * (K + 1);
-    for (int c = tid; c <= j; c += kBT) pp[c] = dot[c];
+    const double *p0 = a.part + int64_t(item - chunk) * a.pstride;  // the stream's first item
+    double *pp = a.part + int64_t(item) * a.pstride;
+    for (int c = dots ? tid : j + tid; c <= j; c += kBT) pp[c] = dot[c];
     __threadfence();
     __syncthreads();
     if (tid == 0) {
@@ -456,10 +475,35 @@ __global__ void __launch_bounds__(kBT, 2) bpass_kernel(BatchArgs a, int ph) {
     if (!s_last) continue;
     __threadfence();
     // ------------------------------------------------------------ last item: reduce + scalar step
-    for (int c = tid; c <= j; c += kBT) {
+    if (dots) {
+      // few columns: several threads a column, each a run of the items, added up in order
+      const int parts = pl.nchunks <= 16 || j >= kBT / 2 ? 1 : j >= kBT / 4 ? 2 : j >= kBT / 8 ? 4 : 8;
+      const int wide = kBT / parts, per = (pl.nchunks + parts - 1) / parts;
+      if (parts == 1) {
+        for (int c = tid; c <= j; c += kBT) dot[c] = sum_strided(p0 + c, pl.nchunks, a.pstride);
+      } else {
+        double *psum = reinterpret_cast<double *>(comb);  // kBT doubles
+        const int c = tid % wide, q0 = (tid / wide) * per;
+        psum[tid] = c <= j ? sum_strided(p0 + int64_t(q0) * a.pstride + c, max(0, min(per, pl.nchunks - q0)), a.pstride)
+                           : 0.0;
+        __syncthreads();
+        if (tid <= j) {
+          double t = 0.0;
+          for (int q = 0; q < parts; ++q) t += psum[q * wide + tid];
+          dot[tid] = t;
+        }
+      }
+    } else {  // the norm alone
       double t = 0.0;
-      for (int q = 0; q < pl.nchunks; ++q) t += __ldcg(a.part + sd.part_off + int64_t(q) * (K + 1) + c);
-      dot[c] = t;
+      for (int q = tid; q < pl.nchunks; q += kBT) t += __ldcg(p0 + int64_t(q) * a.pstride + j);
+      t = warp_sum(t);
+      if (lane == 0) nred[warp] = t;
+      __syncthreads();
+      if (tid == 0) {
+        t = 0.0;
+        for (int wq = 0; wq < kBW; ++wq) t += nred[wq];
+        dot[j] = t;
+      }
     }
     __syncthreads();
     if (mode == PASS_A) {
@@ -546,9 +590,20 @@ __global__ void append_kernel(BatchArgs a) {
     S *Vs = static_cast<S *>(a.V) + sd.v_off;
     const float *w = a.W + sd.w_off;
     const S *x = static_cast<const S *>(a.x[sidx]);
-    for (int64_t rr = r0 + threadIdx.x; rr < r1; rr += blockDim.x) {
-      const float v = first ? ((rr < sd.n) ? float(to_c(x[rr])) : 0.f) : w[rr];
-      Vs[((rr >> 5) * K + j) * kTile + (rr & 31)] = Store<S>::from(v * sc);
+    // four rows a thread: one 16-byte (BF16: 8-byte) store per lane into the column's 32-row segment
+    const bool xv = !first || ((reinterpret_cast<uintptr_t>(x) & (4 * sizeof(S) - 1)) == 0);
+#pragma unroll 2
+    for (int64_t rr = r0 + 4 * int64_t(threadIdx.x); rr < r1; rr += 4 * blockDim.x) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (!first) v = *reinterpret_cast<const float4 *>(w + rr);
+      else if (xv && rr + 4 <= sd.n) v = ld4(x + rr);
+      else {
+        if (rr < sd.n) v.x = float(to_c(x[rr]));
+        if (rr + 1 < sd.n) v.y = float(to_c(x[rr + 1]));
+        if (rr + 2 < sd.n) v.z = float(to_c(x[rr + 2]));
+        if (rr + 3 < sd.n) v.w = float(to_c(x[rr + 3]));
+      }
+      st4(Vs + ((rr >> 5) * K + j) * kTile + (rr & 31), make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc));
     }
   }
 }
@@ -560,7 +615,7 @@ using namespace foa;
 using namespace foa::bt;
 
 struct foa_dmd_batch {
-  int S = 0, dtype = 0, sms = 0;
+  int S = 0, dtype = 0, sms = 0, pstride = 0;
   cudaStream_t stream = nullptr;
   double tol = 0.0;
   std::vector<StreamDesc> sd_host;
@@ -581,16 +636,14 @@ static void batch_free(foa_dmd_batch *b) {
     if (p) cudaFree(p);
 }
 
-// the largest number of work items a pass of this stream can have (over every basis size j)
+// the largest number of work items of kItemBytesMax a pass of this stream can have (over every basis size j)
 static int32_t max_items(int32_t ntiles, int32_t kmax, int es) {
   int32_t best = 1;
   for (int j = 0; j < kmax; ++j) {
     const int R = stage_tiles(j);
     const int64_t nstages = (ntiles + R - 1) / R;
     const int64_t stage_bytes = int64_t(R) * kTile * (j > 0 ? j : 1) * es;
-    int64_t cs = kItemBytes / stage_bytes;
-    if (cs > kItemStages) cs = kItemStages;
-    if (cs < 1) cs = 1;
+    const int64_t cs = item_stages(kItemBytesMax, stage_bytes);
     const int64_t nc = (nstages + cs - 1) / cs;
     if (nc > best) best = int32_t(nc);
   }
@@ -618,7 +671,8 @@ extern "C" int foa_dmd_batch_create(int32_t S, const int64_t *n, const int32_t *
   b->stream = static_cast<cudaStream_t>(o.cuda_stream);
   b->tol = o.breakdown_tol > 0.0 ? o.breakdown_tol : default_tol(dtype);
   const int es = dtype_size(dtype);
-  int64_t voff = 0, woff = 0, moff = 0, vecoff = 0, poff = 0;
+  int64_t voff = 0, woff = 0, moff = 0, vecoff = 0, items = 0;
+  int pstride = 0;
   b->sd_host.resize(S);
   for (int s = 0; s < S; ++s) {
     StreamDesc &d = b->sd_host[s];
@@ -636,11 +690,14 @@ extern "C" int foa_dmd_batch_create(int32_t S, const int64_t *n, const int32_t *
     moff += int64_t(d.kmax) * d.kmax;
     d.vec_off = vecoff;
     vecoff += 3 * int64_t(d.kmax);
-    d.max_chunks = max_items(d.ntiles, d.kmax, es);
-    d.part_off = poff;
-    poff += int64_t(d.max_chunks) * (d.kmax + 1);
-    d.pad = 0;
+    items += max_items(d.ntiles, d.kmax, es);
+    if (d.kmax + 1 > pstride) pstride = d.kmax + 1;
   }
+  // Items of a pass: a stream's are as many as max_items where they have kItemStages stages or
+  // kItemBytesMax bytes, else at most 1.5 x its share of kItemsPerCta a CTA, plus one (a stage is at most
+  // half of kItemBytesMin, so whole stages fill two thirds of the goal).
+  items += 3 * int64_t(sms) * kItemsPerCta + S;
+  b->pstride = pstride;
   cudaError_t e = cudaSuccess;
 #define BAL(p, bytes)                                         \
   do {                                                        \
@@ -659,7 +716,7 @@ extern "C" int foa_dmd_batch_create(int32_t S, const int64_t *n, const int32_t *
   BAL(b->H, size_t(moff) * 8);
   BAL(b->B, size_t(moff) * 8);
   BAL(b->vec, size_t(vecoff) * 8);
-  BAL(b->part, size_t(poff) * 8);
+  BAL(b->part, size_t(items) * pstride * 8);
 #undef BAL
   if (e == cudaSuccess) e = cudaMemcpy(b->sd, b->sd_host.data(), sizeof(StreamDesc) * S, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(b->st, 0, sizeof(BState) * S);
@@ -699,6 +756,8 @@ extern "C" int foa_dmd_batch_push(foa_dmd_batch_t *b, const void *const *x_dev, 
   a.B = b->B;
   a.vec = b->vec;
   a.part = b->part;
+  a.pstride = b->pstride;
+  a.ctas = 2 * b->sms;
   a.x = x_dev;
   a.h_last = h_last_dev;
   a.tol = b->tol;
