@@ -3,9 +3,10 @@
 //   BLK_A  (one pass over V)  C1 = V^T X_b and ||psi_k||^2
 //   BLK_B  (one pass over V)  W = X_b - V C1,  C2 = V^T W,  C = C1 + C2
 //   BLK_C  (one pass over V)  W = W - V C2,    G = W^T W, then G = R1^T R1 (Cholesky, FP64)
-//   BLK_Q1 (rows of W only)   W1 = W R1^-1 (FP64), G2 = W1^T W1 = R2^T R2, R = R2 R1, breakdown test,
-//                             beta block column [C; R], Hbar columns by forward substitution
-//   BLK_Q2 (rows of W only)   Q = W1 R2^-1 -> V columns j .. j+P-1
+//   blockq1 (rows of W only)  W1 = W R1^-1 (FP64), G2 = W1^T W1 = R2^T R2, R = R2 R1, breakdown test,
+//                             beta block column [C; R]; without the rows where R1 is well conditioned
+//   blockh                    Hbar columns by forward substitution, one warp per row
+//   blockq2 (rows of W only)  Q = W R^-1 -> V columns j .. j+P-1
 // V is read three times per block instead of three times per snapshot.  The three passes over V
 // are block_pass.cuh (register-held fragments, packed FP32 FMAs, per-CTA FP64 partials and a
 // deterministic two-level cross-CTA reduction; FP32/BF16 storage).  From the Gram matrix on, the
@@ -21,63 +22,78 @@
 namespace foa {
 namespace blk {
 
-// W1 = W R1^-1 on the leading m1 columns (FP64), G2 = W1^T W1 (per CTA partials), and in the last CTA:
-// R2, R = R2 R1, the breakdown test, the beta block column, the Hbar columns, the device state.
+// The second Cholesky step and the scalar part of the block.  W1 = W R1^-1 on the leading m1 columns
+// (FP64, by reciprocals), G2 = W1^T W1, and in the last CTA: R2, R = R2 R1, the breakdown test, the
+// beta block column, the device state.  The rows cost 20 FP64 operations each at 2 a clock and SM; where
+// R1 is well conditioned (kWellKappa) R2 = I is as good and one CTA does the scalar part alone.  (With
+// divisions, the rows always, and the Hbar columns in the last CTA: 502 us a block at n = 4194304.)
 template <int P>
 __global__ void __launch_bounds__(256) blockq1_kernel(BlockArgs a, foa_dmd_push_info *info_out) {
-  __shared__ double red[256 * P * P];
-  __shared__ double dot[P * P];
+  constexpr int NG = P * (P + 1) / 2;
+  __shared__ double red[8 * NG];
+  __shared__ double dot[NG];
   __shared__ volatile int sflag[4];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (!a.st->active) return;
   BlockState *bs = a.bs;
   const int m1 = __ldcg(&bs->m1);
-  double R1[P * P];
+  const bool well = __ldcg(&bs->well) != 0;
+  if (well) {
+    if (blockIdx.x != 0) return;
+  } else {
+    double R1[P * P], iv[P];
 #pragma unroll
-  for (int i = 0; i < P * P; ++i) R1[i] = __ldcg(&bs->R1[(i % P) + (i / P) * kMaxP]);
-  double g[P * P];
+    for (int i = 0; i < P * P; ++i) R1[i] = __ldcg(&bs->R1[(i % P) + (i / P) * kMaxP]);
 #pragma unroll
-  for (int i = 0; i < P * P; ++i) g[i] = 0.0;
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t r = int64_t(blockIdx.x) * blockDim.x + tid; r < a.nrows; r += stride) {
-    float w[P];
+    for (int c = 0; c < P; ++c) iv[c] = c < m1 ? 1.0 / R1[c + c * P] : 0.0;
+    double g[NG];
 #pragma unroll
-    for (int k = 0; k < P; ++k) w[k] = a.W[int64_t(k) * a.nrows + r];
-    // w1_c = (w_c - sum_{k<c} w1_k R1_{k,c}) / R1_{c,c}, in FP64 for the small triangular solve
-    double w1[P];
+    for (int i = 0; i < NG; ++i) g[i] = 0.0;
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t r = int64_t(blockIdx.x) * blockDim.x + tid; r < a.nrows; r += stride) {
+      double w1[P];
 #pragma unroll
-    for (int c = 0; c < P; ++c) {
-      double t = w[c];
+      for (int c = 0; c < P; ++c) {
+        double t = a.W[int64_t(c) * a.nrows + r];
 #pragma unroll
-      for (int k = 0; k < c; ++k) t -= w1[k] * R1[k + c * P];
-      w1[c] = (c < m1) ? t / R1[c + c * P] : 0.0;
+        for (int k = 0; k < c; ++k) t -= w1[k] * R1[k + c * P];
+        w1[c] = t * iv[c];
+      }
+      int q = 0;
+#pragma unroll
+      for (int k = 0; k < P; ++k)
+#pragma unroll
+        for (int l = k; l < P; ++l, ++q) g[q] += w1[k] * w1[l];
     }
 #pragma unroll
-    for (int c = 0; c < P; ++c) a.W64[int64_t(c) * a.nrows + r] = w1[c];
-#pragma unroll
-    for (int k = 0; k < P; ++k)
-#pragma unroll
-      for (int l = 0; l < P; ++l) g[k + l * P] += w1[k] * w1[l];
+    for (int i = 0; i < NG; ++i) {
+      const double t = warp_sum(g[i]);
+      if (lane == 0) red[warp * NG + i] = t;
+    }
+    __syncthreads();
+    if (tid < NG) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += red[w * NG + tid];
+      dot[tid] = t;
+    }
+    __syncthreads();
+    if (!grid_reduce<256>(a.partials, a.gpart, a.gcount, &bs->ticket[3], NG, dot, NG, sflag + 2, tid)) return;
   }
-#pragma unroll
-  for (int i = 0; i < P * P; ++i) red[tid * P * P + i] = g[i];
-  __syncthreads();
-  if (tid < P * P) {
-    double t = 0.0;
-    for (int i = 0; i < 256; ++i) t += red[i * P * P + tid];
-    dot[tid] = t;
-  }
-  __syncthreads();
-  if (!grid_reduce<256>(a.partials, a.gpart, a.gcount, &bs->ticket[3], P * P, dot, P * P, sflag + 2, tid)) return;
   // ---------------- the last CTA
   const int j = a.j;
   const int K = a.kmax;
   if (tid == 0) {
     double G2[kMaxP * kMaxP];
     for (int i = 0; i < kMaxP * kMaxP; ++i) G2[i] = 0.0;
-    for (int k = 0; k < m1; ++k)
-      for (int l = 0; l < m1; ++l) G2[k + l * kMaxP] = dot[k + l * P];
-    const int m = m1 > 0 ? chol_up(m1, G2, bs->R2) : 0;
+    int m = m1, q = 0;
+    if (well) {
+      for (int i = 0; i < kMaxP * kMaxP; ++i) bs->R2[i] = (i % (kMaxP + 1) == 0) ? 1.0 : 0.0;
+    } else {
+      for (int k = 0; k < P; ++k)
+        for (int l = k; l < P; ++l, ++q)
+          if (l < m1) G2[k + l * kMaxP] = G2[l + k * kMaxP] = dot[q];
+      m = m1 > 0 ? chol_up(m1, G2, bs->R2) : 0;
+    }
     // R = R2 R1: rows r < m for every column c (columns past the factored block keep their
     // coefficients on the factored directions)
     for (int i = 0; i < kMaxP * kMaxP; ++i) bs->R[i] = 0.0;
@@ -118,24 +134,14 @@ __global__ void __launch_bounds__(256) blockq1_kernel(BlockArgs a, foa_dmd_push_
     for (int r = tid; r <= i; r += blockDim.x) a.B[j + r + int64_t(col) * K] = bs->R[r + i * kMaxP];
   }
   __syncthreads();
-  // Hbar columns by forward substitution, one new snapshot after the other
+  // results of the columns (the Hbar columns themselves: blockh_kernel)
   const int ncols = nc + ((status == FOA_DMD_EBREAKDOWN) ? 1 : 0);
-  for (int i = 0; i < ncols; ++i) {
-    const int jc = j - 1 + i, jj = j + i;
-    const double bjj = a.B[jc + int64_t(jc) * K];
-    for (int r = tid; r < jj; r += blockDim.x) {
-      const double brc = (r < j) ? __ldcg(a.C + int64_t(i) * K + r) : bs->R[(r - j) + i * kMaxP];
-      const int l0 = r == 0 ? 0 : r - 1;
-      double acc = 0.0;
-      for (int l = l0; l <= jc - 1; ++l) acc += a.H[r + int64_t(l) * K] * a.B[l + int64_t(jc) * K];
-      a.H[r + int64_t(jc) * K] = (brc - acc) / bjj;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      const double sub = (i < nc) ? bs->R[i + i * kMaxP] / bjj : 0.0;
-      a.H[jj + int64_t(jc) * K] = sub;
+  if (tid == 0) {
+    tri_inv(nc, bs->R, bs->Rinv);
+    for (int i = 0; i < ncols; ++i) {
+      const double bjj = i == 0 ? a.B[int64_t(j - 1) * (K + 1)] : bs->R[(i - 1) * (kMaxP + 1)];
       foa_dmd_push_info inf;
-      inf.h_last = sub;
+      inf.h_last = (i < nc) ? bs->R[i + i * kMaxP] / bjj : 0.0;
       inf.indicator = __longlong_as_double(0x7ff8000000000000ll);
       inf.x_norm = bs->xnorm[i];
       inf.q = j + ((i < nc) ? i + 1 : i);
@@ -143,7 +149,6 @@ __global__ void __launch_bounds__(256) blockq1_kernel(BlockArgs a, foa_dmd_push_
       if (info_out) info_out[i] = inf;
       a.st->info = inf;
     }
-    __syncthreads();
   }
   if (tid == 0) {
     DevState *st = a.st;
@@ -163,30 +168,146 @@ __global__ void __launch_bounds__(256) blockq1_kernel(BlockArgs a, foa_dmd_push_
   }
 }
 
-// Q = W1 R2^-1 -> V columns j .. j+ncommit-1 (row-tiled), rows beyond n zero
+// Hbar columns j-1 .. j+P-2 by forward substitution from beta_{:,2:} = Hbar beta (Eq. matmulhbeta),
+// Hbar_{r,jc} = (beta_{r,jc+1} - sum_{l<jc} Hbar_{r,l} beta_{l,jc}) / beta_{jc,jc}: a row needs only its
+// own entries, so each warp takes a row through all new columns.
+template <int P>
+__global__ void __launch_bounds__(256) blockh_kernel(BlockArgs a) {
+  if (!a.st->active) return;
+  const BlockState *bs = a.bs;
+  const int nc = __ldcg(&bs->ncommit), status = __ldcg(&bs->status);
+  const int ncols = nc + ((status == FOA_DMD_EBREAKDOWN) ? 1 : 0);
+  const int j = a.j, K = a.kmax, lane = threadIdx.x & 31;
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (r >= j + ncols) return;
+  const int l0 = r == 0 ? 0 : r - 1;
+  double acc[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) acc[i] = 0.0;
+  for (int l = l0 + lane; l <= j - 2; l += 32) {
+    const double h = a.H[r + int64_t(l) * K];
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+      if (i < ncols) acc[i] += h * a.B[l + int64_t(j - 1 + i) * K];
+  }
+  double hn[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    hn[i] = 0.0;
+    if (i >= ncols) continue;
+    const int jc = j - 1 + i, jj = j + i;
+    const double bjj = a.B[jc + int64_t(jc) * K];
+    double t = warp_sum(acc[i]);
+#pragma unroll
+    for (int q = 0; q < i; ++q)
+      if (j - 1 + q >= l0) t += hn[q] * a.B[j - 1 + q + int64_t(jc) * K];
+    if (r < jj) {
+      const double brc = (r < j) ? __ldcg(a.C + int64_t(i) * K + r) : bs->R[(r - j) + i * kMaxP];
+      hn[i] = (brc - t) / bjj;
+    } else if (r == jj) {
+      hn[i] = (i < nc) ? bs->R[i + i * kMaxP] / bjj : 0.0;
+    }
+    if (lane == 0 && r <= jj) a.H[r + int64_t(jc) * K] = hn[i];
+  }
+}
+
+// Q = W R^-1 -> V columns j .. j+ncommit-1 (row-tiled), rows beyond n zero.  A thread takes four rows
+// (16-byte accesses).  Where R1 is well conditioned the products with R^-1 are formed in FP32 pairs
+// (each entry of R^-1 as the sum of two floats, exact products and sums by fma and two-sum): 2^-45
+// of sum |w_k r_kc| <= 512 |q_c| per entry, far below the rounding to storage that follows, at FP32's
+// rate; otherwise by two FP64 substitutions.  (FP64 with divisions: 323 us a block at n = 4194304; block push of 256 snapshots there 149 -> 100 ms with the changes here.)
 template <typename S, int P>
-__global__ void blockq2_kernel(BlockArgs a) {
+__global__ void __launch_bounds__(256) blockq2_kernel(BlockArgs a) {
   if (!a.st->active) return;
   const BlockState *bs = a.bs;
   const int nc = __ldcg(&bs->ncommit);
   if (nc == 0) return;
-  double R2[P * P];
-#pragma unroll
-  for (int i = 0; i < P * P; ++i) R2[i] = __ldcg(&bs->R2[(i % P) + (i / P) * kMaxP]);
+  const bool well = __ldcg(&bs->well) != 0;
   S *V = static_cast<S *>(const_cast<void *>(a.V));
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < a.nrows; r += stride) {
-    double q[P];
+  const int64_t stride = 4 * int64_t(gridDim.x) * blockDim.x;
+  const int64_t first = 4 * (int64_t(blockIdx.x) * blockDim.x + threadIdx.x);
+  auto load = [&](int64_t r, float (&w)[P][4]) {
 #pragma unroll
-    for (int c = 0; c < P; ++c) {
-      double t = a.W64[int64_t(c) * a.nrows + r];
+    for (int k = 0; k < P; ++k) *reinterpret_cast<float4 *>(w[k]) = *reinterpret_cast<const float4 *>(a.W + int64_t(k) * a.nrows + r);
+  };
+  auto store = [&](int64_t r, int c, const float (&q)[4]) {
+    float4 v = make_float4(q[0], q[1], q[2], q[3]);
+    if (r + 4 > a.n) {
+      if (r >= a.n) v.x = 0.f;
+      if (r + 1 >= a.n) v.y = 0.f;
+      if (r + 2 >= a.n) v.z = 0.f;
+      if (r + 3 >= a.n) v.w = 0.f;
+    }
+    st4(V + ((r >> 5) * a.kmax + a.j + c) * kTile + (r & 31), v);
+  };
+  if (well) {
+    float rh[P][P], rl[P][P];
 #pragma unroll
-      for (int k = 0; k < c; ++k) t -= q[k] * R2[k + c * P];
-      q[c] = t / R2[c + c * P];
+    for (int c = 0; c < P; ++c)
+#pragma unroll
+      for (int k = 0; k <= c; ++k) {
+        const double v = __ldcg(&bs->Rinv[k + c * kMaxP]);
+        rh[k][c] = float(v);
+        rl[k][c] = float(v - double(rh[k][c]));
+      }
+    for (int64_t r = first; r < a.nrows; r += stride) {
+      float w[P][4];
+      load(r, w);
+#pragma unroll
+      for (int c = 0; c < P; ++c) {
+        float q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          float s = __fmul_rn(w[0][u], rh[0][c]);
+          float e = fmaf(w[0][u], rl[0][c], fmaf(w[0][u], rh[0][c], -s));
+#pragma unroll
+          for (int k = 1; k <= c; ++k) {
+            const float p = __fmul_rn(w[k][u], rh[k][c]);
+            const float pe = fmaf(w[k][u], rl[k][c], fmaf(w[k][u], rh[k][c], -p));
+            const float t = __fadd_rn(s, p), bb = __fsub_rn(t, s);
+            e = __fadd_rn(e, __fadd_rn(pe, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(p, bb))));
+            s = t;
+          }
+          q[u] = __fadd_rn(s, e);
+        }
+        if (c < nc) store(r, c, q);
+      }
+    }
+    return;
+  }
+  double R1[P * P], R2[P * P], i1[P], i2[P];
+#pragma unroll
+  for (int i = 0; i < P * P; ++i) {
+    R1[i] = __ldcg(&bs->R1[(i % P) + (i / P) * kMaxP]);
+    R2[i] = __ldcg(&bs->R2[(i % P) + (i / P) * kMaxP]);
+  }
+#pragma unroll
+  for (int c = 0; c < P; ++c) {
+    i1[c] = c < nc ? 1.0 / R1[c + c * P] : 0.0;
+    i2[c] = c < nc ? 1.0 / R2[c + c * P] : 0.0;
+  }
+  for (int64_t r = first; r < a.nrows; r += stride) {
+    float w[P][4], q[P][4];
+    load(r, w);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      double w1[P], x[P];
+#pragma unroll
+      for (int c = 0; c < P; ++c) {
+        double t = w[c][u];
+#pragma unroll
+        for (int k = 0; k < c; ++k) t -= w1[k] * R1[k + c * P];
+        w1[c] = t * i1[c];
+        t = w1[c];
+#pragma unroll
+        for (int k = 0; k < c; ++k) t -= x[k] * R2[k + c * P];
+        x[c] = t * i2[c];
+        q[c][u] = float(x[c]);
+      }
     }
 #pragma unroll
     for (int c = 0; c < P; ++c)
-      if (c < nc) V[((r >> 5) * a.kmax + a.j + c) * kTile + (r & 31)] = Store<S>::from(float(r < a.n ? q[c] : 0.0));
+      if (c < nc) store(r, c, q[c]);
   }
 }
 
@@ -214,7 +335,6 @@ namespace {
 
 struct BlockWork {
   float *W = nullptr;
-  double *W64 = nullptr;
   double *C1 = nullptr, *C = nullptr;
   BlockState *bs = nullptr;
   foa_dmd_push_info *info = nullptr;
@@ -281,7 +401,6 @@ int enqueue_block(foa_dmd *h, BlockWork &bw, const void *X, int64_t ldx, foa_dmd
   a.X = X;
   a.ldx = ldx;
   a.W = bw.W;
-  a.W64 = bw.W64;
   a.C1 = bw.C1;
   a.C = bw.C;
   a.partials = h->partials;
@@ -322,6 +441,7 @@ int enqueue_block(foa_dmd *h, BlockWork &bw, const void *X, int64_t ldx, foa_dmd
   if (e == cudaSuccess) {
     const int g = h->sms * 4;
     blockq1_kernel<P><<<g, 256, 0, s>>>(a, info_out);
+    blockh_kernel<P><<<(j + P + 7) / 8, 256, 0, s>>>(a);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
@@ -330,7 +450,7 @@ int enqueue_block(foa_dmd *h, BlockWork &bw, const void *X, int64_t ldx, foa_dmd
     else blockq2_kernel<__nv_bfloat16, P><<<h->sms * 4, 256, 0, s>>>(a);
     e = cudaGetLastError();
   }
-  h->launches += 3;  // prep, Cholesky QR, Q into V
+  h->launches += 4;  // prep, Cholesky QR, Hbar, Q into V
   return cuda_status(e);
 }
 
@@ -349,7 +469,6 @@ extern "C" int foa_dmd_push_block(foa_dmd_t *h, const void *X_dev, int32_t p, in
   if (h->stopped_host) return FOA_DMD_ESTOPPED;
   BlockWork bw;
   cudaError_t e = cudaMalloc(&bw.W, size_t(kMaxP) * h->nrows * 4);
-  if (e == cudaSuccess) e = cudaMalloc(&bw.W64, size_t(kMaxP) * h->nrows * 8);
   if (e == cudaSuccess) e = cudaMalloc(&bw.C1, size_t(kMaxP) * h->kmax * 8);
   if (e == cudaSuccess) e = cudaMalloc(&bw.C, size_t(kMaxP) * h->kmax * 8);
   if (e == cudaSuccess) e = cudaMalloc(&bw.bs, sizeof(BlockState));
@@ -419,7 +538,6 @@ extern "C" int foa_dmd_push_block(foa_dmd_t *h, const void *X_dev, int32_t p, in
   }
   cudaStreamSynchronize(h->stream);
   cudaFree(bw.W);
-  cudaFree(bw.W64);
   cudaFree(bw.C1);
   cudaFree(bw.C);
   cudaFree(bw.bs);
