@@ -22,6 +22,16 @@ static inline int64_t align_up(int64_t v, int64_t a) { return (v + a - 1) / a * 
 
 int max_kmax_for(int dtype) { return dtype == FOA_DMD_F64 ? 384 : kMaxK; }
 
+// FP64 stages are larger: with 128 rows and more the row sweep needs no combine over column groups, and
+// what is done once per row weighs less against the FP64 pipes' 64 cycles an instruction.  Two CTAs
+// per SM overlap one's barriers and row ends with the other's products.  (32 KB, one CTA per SM: 108 ms for
+// 96 pushes of 1048576 values, now 73 ms.)
+Geometry default_geometry(int dtype) {
+  Geometry g;
+  if (dtype == FOA_DMD_F64) g.stage_bytes = 48 * 1024;
+  return g;
+}
+
 // Shared-memory layout and grid of one streaming pass (the launch geometry depends only on the
 // dtype, the pass kind, jcap and n, so identical pushes always get identical launches).
 bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n, int ntiles, int sms, PassArgs &a,
@@ -56,9 +66,10 @@ bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n,
   const int64_t comb_bytes = lag ? 2 * kConsumers * 8 : kConsumers * 8;
   const int64_t other = ws_bytes + vnew_bytes + cf_bytes + cf2_bytes + align_up(int64_t(jcap + 2) * 8, 16) +
                         comb_bytes + kConsumers * 8 + 2 * kMaxSlots * 8 + 64;
-  // two CTAs per SM for FP32/BF16 while two slots fit in half the shared memory; otherwise one CTA
-  // per SM with a deeper ring
-  const bool two = (cs == 4) &&
+  // two CTAs per SM while two slots fit in half the shared memory (FP64: and while the kernel's registers
+  // do, pass_min_blocks); otherwise one CTA per SM with a deeper ring
+  const bool regs = cs == 4 || (!lag && (mode == PASS_C || mode == PASS_FIRST || pass_nc_for(jcap) <= 16));
+  const bool two = regs &&
                    (2 * slot_bytes + other <= g.smem_budget2) && g.max_ctas_per_sm >= 2;
   const int64_t budget = two ? g.smem_budget2 : g.smem_budget;
   const int64_t inflight = two ? g.inflight_bytes / 2 : g.inflight_bytes;
@@ -345,7 +356,7 @@ extern "C" int foa_dmd_create(int64_t n, int32_t k_max, int32_t dtype, const foa
   h->sms = sms;
   h->stream = static_cast<cudaStream_t>(h->opts.cuda_stream);
   h->tol = h->opts.breakdown_tol > 0.0 ? h->opts.breakdown_tol : default_tol(dtype);
-  h->geom = Geometry();
+  h->geom = default_geometry(dtype);
   rc = alloc_handle(h);
   if (rc) {
     free_handle_buffers(h);

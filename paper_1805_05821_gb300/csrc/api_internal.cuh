@@ -112,6 +112,7 @@ int sync_state(foa_dmd *h, foa_dmd_push_info *info);
 int check_device(int *sms);
 double default_tol(int dtype);
 int max_kmax_for(int dtype);
+Geometry default_geometry(int dtype);
 bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n, int ntiles, int sms, PassArgs &a,
                     int &grid);
 int launch_pass_h(foa_dmd *h, int mode, int jcap, const void *x, const double *coef, bool batch,

@@ -91,6 +91,7 @@ extern "C" int foa_dmd_push_noalloc(int64_t n, int32_t k_max, int32_t dtype, voi
   h.sms = sms;
   h.stream = s;
   h.tol = breakdown_tol > 0.0 ? breakdown_tol : default_tol(dtype);
+  h.geom = default_geometry(dtype);
   h.V = V;
   h.w = w_dev;
   h.H = Hbar;

@@ -274,11 +274,11 @@ __device__ __forceinline__ void drain(const PassArgs &a, uint64_t *full) {
     if (blockIdx.x + k * gridDim.x < a.nstages) mbar_wait(&full[k], 0);
 }
 
-// Two CTAs per SM for the FP32/BF16 forms while the column accumulators fit (NC <= 48, i.e.
-// j <= 384): one CTA's barrier phases then overlap the other's compute.
+// Two CTAs per SM while the column accumulators fit (FP32/BF16: NC <= 48, i.e. j <= 384; FP64: NC <= 16,
+// j <= 128): one CTA's barrier phases then overlap the other's compute.
 template <typename S, int NC>
 constexpr int pass_min_blocks() {
-  return (sizeof(typename Compute<S>::T) == 4 && NC <= 48) ? 2 : 1;
+  return NC <= (sizeof(typename Compute<S>::T) == 4 ? 48 : 16) ? 2 : 1;
 }
 
 template <typename S, int MODE, int NC>
