@@ -46,7 +46,11 @@ bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n,
   if (jj == 0) {
     R = kMaxR;
   } else {
-    while (R * 2 <= kMaxR && (R * 2) * tile_bytes <= g.stage_bytes) R *= 2;
+    // FP32/BF16 passes with column dots: up to the register-held kernel's row pairs, unless the
+    // shared-memory form is asked for
+    const bool held = cs == 4 && g.variant == 0 && (mode == PASS_A || mode == PASS_B || mode == PASS_B2);
+    const int max_r = held ? kFusedMaxR : kMaxR;
+    while (R * 2 <= max_r && (R * 2) * tile_bytes <= g.stage_bytes) R *= 2;
   }
   // FP64 storage is bound by the FP64 pipes (2 FMAs a clock and SM): few tiles are spread over all SMs in
   // smaller stages, down to 8 KB.  (n = 4096, 11 pushes and the solve: 1.67 -> 1.30 ms.  FP32 stages

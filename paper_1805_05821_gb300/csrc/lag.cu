@@ -47,7 +47,7 @@ static cudaError_t launch_lag_t(int mode, int nc, const PassArgs &a, int grid, c
   if constexpr (sizeof(typename Compute<S>::T) == 4) {
     // FP32/BF16: stages of one or two tiles held in registers, else the warp-specialised kernel
     // (row and column sweeps on different warps)
-    const int fc = fused_columns(a);
+    const int fc = fused_columns(a, 2);
     if (fc == 16) return launch_lag_fused_one<S, 16>(a, grid, s);
     if (fc == 24) return launch_lag_fused_one<S, 24>(a, grid, s);
     if (fc == 32) return launch_lag_fused_one<S, 32>(a, grid, s);

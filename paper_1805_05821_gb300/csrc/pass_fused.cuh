@@ -1,17 +1,21 @@
-// Streaming pass with the stage held in registers (FP32/BF16 storage, passes A, B and B2 when a
-// pipeline stage is one or two 32-row tiles, i.e. the wide-basis part of a run).
+// Streaming pass with the stage held in registers (FP32/BF16 storage, passes A, B and B2).
 //
-// A thread owns a fixed pair of adjacent rows of every stage and a fixed group of columns
-// (16 or 32 threads share a column group).  Per stage it loads its V fragment (2 rows x FC
+// A thread owns a fixed pair of adjacent rows of every stage (R tiles, R <= 16) and a fixed group of
+// at most 32 columns (16 R threads share a column group).  Per stage it loads its V fragment (2 rows x FC
 // columns) into registers once; from the registers,
 //   row sweep:     partial sums of the GEMV-N for its two rows, combined across the column groups
 //                  through shared memory, the new w of the stage's rows (as pass_kernel);
 //   column sweep:  its columns' dot products with the two new w values, one FP32 accumulator
 //                  per column, folded every 16 stages (32 products per lane) by a shuffle tree
-//                  over the threads of the column group into the CTA's FP64 dot vector.
+//                  over the threads of the column group into FP64 (the CTA's dot vector where a group lies
+//                  inside a warp, a sum per warp otherwise).
 // There is no producer warp: the CTA is the eight compute warps (two CTAs of 256 threads per SM,
 // up to 128 registers a thread for the fragment), and one elected thread refills a ring slot as
 // soon as the first CTA barrier of the stage shows every thread holding its fragment.
+// A stage costs a CTA about 1700 cycles of barriers and latency whatever it holds, so it is filled:
+// 32 KB, R j <= 256 columns of tiles in FP32, 512 in BF16, down to j = 1.  (With stages of one or two tiles
+// only, and the warp-specialised kernel for the rest, BF16 ran at 1.3 TB/s at j = 16, 2.3 at j = 80, n = 8388608,
+// and FP32 at 3.8 TB/s at j = 16.  160 pushes of 2097152 BF16 values: 58.0 -> 49.5 ms.)
 // The cross-CTA reduction and the scalar step are pass_epilogue.
 #pragma once
 #include "pass.cuh"
@@ -19,10 +23,10 @@
 namespace foa {
 
 // Columns per thread of the register-held pass for this launch (16, 24 or 32), or 0 when the stage
-// is wider than two tiles, the column groups would exceed 32 columns, or the launch asks for the
+// is wider than max_r tiles, the column groups would exceed 32 columns, or the launch asks for the
 // shared-memory form (PassArgs::variant).
-inline int fused_columns(const PassArgs &a) {
-  if (a.variant != 0 || a.R > 2) return 0;
+inline int fused_columns(const PassArgs &a, int max_r = kFusedMaxR) {
+  if (a.variant != 0 || a.R > max_r) return 0;
   const int G1 = kConsumers / (a.R * (kTile / 2));
   const int cpg = (((a.jcap + G1 - 1) / G1) + 3) & ~3;
   return cpg <= 16 ? 16 : cpg <= 24 ? 24 : cpg <= 32 ? 32 : 0;
@@ -44,7 +48,7 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
   float *cf = reinterpret_cast<float *>(smem + a.off_coef);    // coefficients, zero padded
   double *dot = reinterpret_cast<double *>(smem + a.off_dot);
   float *comb = reinterpret_cast<float *>(smem + a.off_comb);  // row-sweep group partials
-  double *nrm = reinterpret_cast<double *>(smem + a.off_norm);
+  double *nrm = reinterpret_cast<double *>(smem + a.off_norm);  // until the norms: [warp][FC] column sums (R >= 4)
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + a.off_bar);
   volatile int *sflag = reinterpret_cast<volatile int *>(full + 2 * kMaxSlots);  // [0] abort [2] last
 
@@ -62,30 +66,33 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
   // the ring's first stages of V before the predecessor is waited for, their base slices after it
   const int jp = prefetch_columns<MODE>(a, st);
   if (tid == kIssuer && jp)
-    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, slots, full);
+    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, backwards<MODE>(jp), slots, full);
   pdl_wait();
   pdl_trigger();
   if (tid == kIssuer && jp)
-    for (int k = 0; k < a.slots; ++k) issue_base<BaseT, kBaseX>(a, bg, k, blockIdx.x + k * gridDim.x, slots, full);
+    for (int k = 0; k < a.slots; ++k)
+      issue_base<BaseT, kBaseX>(a, bg, k, blockIdx.x + k * gridDim.x, backwards<MODE>(jp), slots, full);
   const int j = st->j;
   if (!st->active || j < 1 || j > a.jcap || (jp && jp != j)) {
     if (tid == kIssuer && jp) drain(a, full);
     return;
   }
+  const bool back = backwards<MODE>(j);
   const bool qr_a = (MODE == PASS_A) && a.form != 0;
   const float cscale = (MODE == PASS_A && !qr_a) ? float(st->inv_bjj) : 1.f;
   // fixed mapping: PF row pairs per full stage (R tiles), G1 column groups of cpg columns
-  const int PF = a.R * (kTile / 2);                   // 16 (R = 1) or 32 (R = 2)
-  const int G1 = kConsumers / PF;                     // 16 or 8
+  const int PF = a.R * (kTile / 2);                   // 16 .. 256
+  const int G1 = kConsumers / PF;                     // 16 .. 1
   const int cpg = (((j + G1 - 1) / G1) + 3) & ~3;     // <= FC (host check)
   // coefficients zero-padded past every group's FC-wide window (G1*cpg + FC <= j + 88 < jcap + 96)
   for (int c = tid; c < G1 * cpg + FC; c += kConsumers) cf[c] = c < j ? static_cast<float>(a.coef[c]) : 0.f;
   for (int c = tid; c <= j; c += kConsumers) dot[c] = 0.0;
+  nrm[tid] = 0.0;
   __syncthreads();
 
   auto issue = [&](int slot, int s) {
-    issue_v<S, BaseT, kBaseX>(a, j, slot, s, slots, full);
-    issue_base<BaseT, kBaseX>(a, bg, slot, s, slots, full);
+    issue_v<S, BaseT, kBaseX>(a, j, slot, s, back, slots, full);
+    issue_base<BaseT, kBaseX>(a, bg, slot, s, back, slots, full);
   };
   if (tid == kIssuer && !jp)
     for (int k = 0; k < a.slots; ++k) issue(k, blockIdx.x + k * gridDim.x);
@@ -105,14 +112,20 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
     nsum = t;
   };
   auto flush = [&]() {
-    // sum over the PF threads of the column group (lanes of one half-warp or one warp)
+    // sum over the PF threads of the column group, or those of them in this warp
 #pragma unroll
     for (int u = 0; u < FC; ++u) {
       float v = cacc[u];
-      if (PF == 32) v += __shfl_xor_sync(0xffffffffu, v, 16);
+      if (PF >= 32) v += __shfl_xor_sync(0xffffffffu, v, 16);
 #pragma unroll
       for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (pr == 0 && u < nc) dot[c0 + u] += static_cast<double>(v);
+      if (u < nc) {
+        if (PF <= 32) {
+          if (pr == 0) dot[c0 + u] += static_cast<double>(v);
+        } else if ((tid & 31) == 0) {
+          nrm[(tid >> 5) * FC + u] += static_cast<double>(v);
+        }
+      }
       cacc[u] = 0.f;
     }
   };
@@ -124,7 +137,7 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
       sflag[0] = 1;
       atomicExch(&st->err, FOA_DMD_ETIMEOUT);
     }
-    const int t0 = s * a.R;
+    const int t0 = stage_at(a, s, back) * a.R;
     const int nt = min(a.R, a.ntiles - t0);
     const int RS = nt * kTile;
     const int64_t r0 = int64_t(t0) * kTile;
@@ -140,10 +153,14 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
 #pragma unroll
       for (int u = 0; u < FC; ++u) v[u] = (has_rows && u < nc) ? ld_pair(vr + (c0 + u) * kTile) : make_float2(0.f, 0.f);
     }
-    float base = 0.f;
-    if (tid < RS) {
-      if (base_bulk) base = to_c(reinterpret_cast<const BaseT *>(sbase + a.base_off)[tid]);
-      else base = (r0 + tid < a.n) ? float(to_c(bg[r0 + tid])) : 0.f;
+    float base[2] = {0.f, 0.f};  // rows tid and tid + 256
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int rr = tid + h * kConsumers;
+      if (rr < RS) {
+        if (base_bulk) base[h] = to_c(reinterpret_cast<const BaseT *>(sbase + a.base_off)[rr]);
+        else base[h] = (r0 + rr < a.n) ? float(to_c(bg[r0 + rr])) : 0.f;
+      }
     }
     // ---------------- row sweep from registers
     if (!qr_a) {
@@ -160,18 +177,20 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
       comb[g * (2 * PF) + row + 1] = b0 + b1;
     }
     named_bar_sync(1, kConsumers);  // every thread holds its fragment: the slot is free
-    if (tid == kIssuer && !sflag[0]) {
-      issue(slot, s + a.slots * gridDim.x);
-    }
-    if (tid < RS) {
-      float acc = 0.f;
-      if (!qr_a)
-        for (int gg = 0; gg < G1; ++gg) acc += comb[gg * (2 * PF) + tid];
-      const float wc = (MODE == PASS_A) ? (base - acc) * cscale : (base - acc);
-      static_cast<float *>(a.w)[r0 + tid] = wc;
-      ws[tid] = wc;
-      if constexpr (MODE == PASS_A) nrm_add(base * base);
-      else if constexpr (MODE == PASS_B2) nrm_add(wc * wc);
+    if (tid == kIssuer && !sflag[0]) issue(slot, s + a.slots * gridDim.x);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int rr = tid + h * kConsumers;
+      if (rr < RS) {
+        float acc = 0.f;
+        if (!qr_a)
+          for (int gg = 0; gg < G1; ++gg) acc += comb[gg * (2 * PF) + rr];
+        const float wc = (MODE == PASS_A) ? (base[h] - acc) * cscale : (base[h] - acc);
+        static_cast<float *>(a.w)[r0 + rr] = wc;
+        ws[rr] = wc;
+        if constexpr (MODE == PASS_A) nrm_add(base[h] * base[h]);
+        else if constexpr (MODE == PASS_B2) nrm_add(wc * wc);
+      }
     }
     named_bar_sync(1, kConsumers);  // ws complete
     // ---------------- column sweep from registers
@@ -186,6 +205,16 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
     }
   }
   flush();
+  if (PF > 32) {  // the warps' sums of each column group, in warp order
+    named_bar_sync(1, kConsumers);
+    for (int c = tid; c < j; c += kConsumers) {
+      const int gc = c / cpg, w0 = gc * (PF / 32);
+      double t = 0.0;
+      for (int w = w0; w < w0 + PF / 32; ++w) t += nrm[w * FC + c - gc * cpg];
+      dot[c] = t;
+    }
+    named_bar_sync(1, kConsumers);
+  }
   nrm[tid] = kNorm ? double(nsum) - double(ncomp) : 0.0;
   pass_epilogue<MODE>(a, st, dot, nrm, sflag, j, tid);
 }
