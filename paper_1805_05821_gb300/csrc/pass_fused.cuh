@@ -1,16 +1,16 @@
-// Streaming pass with the stage held in registers (FP32/BF16 storage, passes A, B and B2).
+// Streaming pass with the stage held in registers (FP32/BF16 storage, passes A, B, C and B2).
 //
 // A thread owns a fixed pair of adjacent rows of every stage (R tiles, R <= 16) and a fixed group of
 // at most 32 columns (16 R threads share a column group).  Per stage it loads its V fragment (2 rows x FC
 // columns) into registers once; from the registers,
 //   row sweep:     partial sums of the GEMV-N for its two rows, combined across the column groups
 //                  through shared memory, the new w of the stage's rows (as pass_kernel);
-//   column sweep:  its columns' dot products with the two new w values, one FP32 accumulator
+//   column sweep (not in pass C):  its columns' dot products with the two new w values, one FP32 accumulator
 //                  per column, folded every 16 stages (32 products per lane) by a shuffle tree
 //                  over the threads of the column group into FP64 (the CTA's dot vector where a group lies
 //                  inside a warp, a sum per warp otherwise).
 // There is no producer warp: the CTA is the eight compute warps (two CTAs of 256 threads per SM,
-// up to 128 registers a thread for the fragment), and one elected thread refills a ring slot as
+// up to 128 registers a thread for the fragment; three with at most 16 columns a thread), and one elected thread refills a ring slot as
 // soon as the first CTA barrier of the stage shows every thread holding its fragment.
 // A stage costs a CTA about 1700 cycles of barriers and latency whatever it holds, so it is filled:
 // 32 KB, R j <= 256 columns of tiles in FP32, 512 in BF16, down to j = 1.  (With stages of one or two tiles
@@ -23,21 +23,22 @@
 namespace foa {
 
 // Columns per thread of the register-held pass for this launch (16, 24 or 32), or 0 when the stage
-// is wider than max_r tiles, the column groups would exceed 32 columns, or the launch asks for the
+// is wider than 16 tiles, the column groups would exceed 32 columns, or the launch asks for the
 // shared-memory form (PassArgs::variant).
-inline int fused_columns(const PassArgs &a, int max_r = kFusedMaxR) {
-  if (a.variant != 0 || a.R > max_r) return 0;
+inline int fused_columns(const PassArgs &a) {
+  if (a.variant != 0 || a.R > kFusedMaxR) return 0;
   const int G1 = kConsumers / (a.R * (kTile / 2));
   const int cpg = (((a.jcap + G1 - 1) / G1) + 3) & ~3;
   return cpg <= 16 ? 16 : cpg <= 24 ? 24 : cpg <= 32 ? 32 : 0;
 }
 
 template <typename S, int MODE, int FC>
-__global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArgs a) {
+__global__ void __launch_bounds__(kConsumers, FC == 16 ? 3 : 2) pass_fused_kernel(const PassArgs a) {
   static_assert(sizeof(typename Compute<S>::T) == 4, "FP32/BF16 storage only");
-  static_assert(MODE == PASS_A || MODE == PASS_B || MODE == PASS_B2, "passes with column dots only");
+  static_assert(MODE == PASS_A || MODE == PASS_B || MODE == PASS_B2 || MODE == PASS_C, "passes over V");
   constexpr bool kBaseX = (MODE == PASS_A);
-  constexpr bool kNorm = (MODE == PASS_A || MODE == PASS_B2);
+  constexpr bool kDots = (MODE != PASS_C);
+  constexpr bool kNorm = (MODE == PASS_A || MODE == PASS_B2 || MODE == PASS_C);
   using BaseT = typename std::conditional<kBaseX, S, float>::type;
 
   extern __shared__ __align__(128) unsigned char smem[];
@@ -101,9 +102,9 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
   const int g = tid / PF, pr = tid % PF;
   const int c0 = g * cpg;
   const int nc = max(0, min(j, c0 + cpg) - c0);       // this thread's columns
-  float cacc[FC];
+  float cacc[kDots ? FC : 1];
 #pragma unroll
-  for (int u = 0; u < FC; ++u) cacc[u] = 0.f;
+  for (int u = 0; u < (kDots ? FC : 1); ++u) cacc[u] = 0.f;
   float nsum = 0.f, ncomp = 0.f;
   auto nrm_add = [&](float v) {
     const float y = v - ncomp;
@@ -113,20 +114,22 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
   };
   auto flush = [&]() {
     // sum over the PF threads of the column group, or those of them in this warp
+    if constexpr (kDots) {
 #pragma unroll
-    for (int u = 0; u < FC; ++u) {
-      float v = cacc[u];
-      if (PF >= 32) v += __shfl_xor_sync(0xffffffffu, v, 16);
+      for (int u = 0; u < FC; ++u) {
+        float v = cacc[u];
+        if (PF >= 32) v += __shfl_xor_sync(0xffffffffu, v, 16);
 #pragma unroll
-      for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (u < nc) {
-        if (PF <= 32) {
-          if (pr == 0) dot[c0 + u] += static_cast<double>(v);
-        } else if ((tid & 31) == 0) {
-          nrm[(tid >> 5) * FC + u] += static_cast<double>(v);
+        for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (u < nc) {
+          if (PF <= 32) {
+            if (pr == 0) dot[c0 + u] += static_cast<double>(v);
+          } else if ((tid & 31) == 0) {
+            nrm[(tid >> 5) * FC + u] += static_cast<double>(v);
+          }
         }
+        cacc[u] = 0.f;
       }
-      cacc[u] = 0.f;
     }
   };
   int since_flush = 0;
@@ -187,25 +190,27 @@ __global__ void __launch_bounds__(kConsumers, 2) pass_fused_kernel(const PassArg
           for (int gg = 0; gg < G1; ++gg) acc += comb[gg * (2 * PF) + rr];
         const float wc = (MODE == PASS_A) ? (base[h] - acc) * cscale : (base[h] - acc);
         static_cast<float *>(a.w)[r0 + rr] = wc;
-        ws[rr] = wc;
+        if constexpr (kDots) ws[rr] = wc;
         if constexpr (MODE == PASS_A) nrm_add(base[h] * base[h]);
-        else if constexpr (MODE == PASS_B2) nrm_add(wc * wc);
+        else if constexpr (MODE == PASS_B2 || MODE == PASS_C) nrm_add(wc * wc);
       }
     }
-    named_bar_sync(1, kConsumers);  // ws complete
+    named_bar_sync(1, kConsumers);  // ws complete, comb free
     // ---------------- column sweep from registers
-    if (has_rows) {
-      const float2 wv = *reinterpret_cast<const float2 *>(ws + row);
+    if constexpr (kDots) {
+      if (has_rows) {
+        const float2 wv = *reinterpret_cast<const float2 *>(ws + row);
 #pragma unroll
-      for (int u = 0; u < FC; ++u) cacc[u] = fmaf(v[u].x, wv.x, fmaf(v[u].y, wv.y, cacc[u]));
-    }
-    if (++since_flush == 16) {  // 32 products per thread and column
-      flush();
-      since_flush = 0;
+        for (int u = 0; u < FC; ++u) cacc[u] = fmaf(v[u].x, wv.x, fmaf(v[u].y, wv.y, cacc[u]));
+      }
+      if (++since_flush == 16) {  // 32 products per thread and column
+        flush();
+        since_flush = 0;
+      }
     }
   }
   flush();
-  if (PF > 32) {  // the warps' sums of each column group, in warp order
+  if (kDots && PF > 32) {  // the warps' sums of each column group, in warp order
     named_bar_sync(1, kConsumers);
     for (int c = tid; c < j; c += kConsumers) {
       const int gc = c / cpg, w0 = gc * (PF / 32);
