@@ -181,6 +181,7 @@ void free_handle_buffers(foa_dmd *h) {
                   h->info_dev, h->stage_x};
   for (void *p : ptrs)
     if (p) cudaFree(p);
+  if (h->pin) cudaFreeHost(h->pin);
   for (auto &e : h->events) {
     cudaEventDestroy(e.start);
     cudaEventDestroy(e.stop);
@@ -195,10 +196,12 @@ void free_handle_buffers(foa_dmd *h) {
 }
 
 int sync_state(foa_dmd *h, foa_dmd_push_info *info) {
-  DevState st;
-  cudaError_t e = cudaMemcpyAsync(&st, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream);
+  // through pinned memory: a copy to pageable memory waits for the stream and is then staged
+  DevState *host = static_cast<DevState *>(h->pin);
+  cudaError_t e = cudaMemcpyAsync(host, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_status(e);
+  const DevState st = *host;
   h->q_host = st.q;
   h->stopped_host = st.stopped != 0;
   if (info) *info = st.info;
@@ -211,7 +214,7 @@ int alloc_handle(foa_dmd *h) {
   const int s = dtype_size(h->dtype), cs = compute_size(h->dtype);
   const int K = h->kmax;
   const int maxgrid = h->sms * 8;
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = cudaHostAlloc(&h->pin, pin_bytes(K), cudaHostAllocDefault);
 #define ALLOC(ptr, bytes)                                  \
   do {                                                     \
     if (e == cudaSuccess) e = cudaMalloc((void **)&(ptr), (bytes)); \

@@ -52,6 +52,7 @@ struct foa_dmd {
   uint32_t *gcount = nullptr;
   foa::DevState *st = nullptr;
   foa_dmd_push_info *info_dev = nullptr;
+  void *pin = nullptr;  // pinned: small results on their way to the host (pin_bytes)
   void *stage_x = nullptr;
   int stage_flip = 0;
   cudaStream_t copy_stream = nullptr;        // host->device snapshot copies (foa_dmd_push_host)
@@ -109,6 +110,9 @@ struct ProfScope {
 };
 
 int cuda_status(cudaError_t e);
+// the device state, or the eigensolve's sorted block, integer scalars and h_{m+1,m}
+inline size_t pin_bytes(int kmax) { return 1024 + size_t(kmax) * 5 * 8; }
+static_assert(sizeof(DevState) <= 1024, "DevState fits pin_bytes");
 int sync_state(foa_dmd *h, foa_dmd_push_info *info);
 int check_device(int *sms);
 double default_tol(int dtype);

@@ -201,7 +201,7 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   if (nsel > m) nsel = m;
   order_kernel<<<1, 512, size_t(m) * 20 + 64, s>>>(a, nsel);
   // roots_setup (start, steps, pair, finish), hqr, flip, invit, vectors, order
-  h->launches += 6 + (m >= kRootMinOrder ? kRootSteps32 + kRootSteps + 3 : 0);
+  h->launches += 6 + (m >= kRootMin32 ? kRootSteps32 : 0) + (m >= kRootMinOrder ? kRootSteps + 3 : 0);
   if (trunc && copied) {
     e = cudaEventRecord(copied, s);
     if (e != cudaSuccess) return cuda_status(e);
@@ -231,14 +231,21 @@ static int run_eig_body(foa_dmd *h, double rank_tol, int nsel, EigOut &res) {
   cudaStream_t s = h->stream;
   rc = enqueue_eig(h, w, s, m, rank_tol, nsel);
   if (rc) return rc;
-  res.out.resize(size_t(OUT_N) * K);
-  int iscv[ISC_N];
-  double hb = 0.0;
-  cudaError_t e = cudaMemcpyAsync(res.out.data(), w->out, res.out.size() * 8, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(iscv, w->isc, sizeof(iscv), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hb, h->H + m + int64_t(m - 1) * K, 8, cudaMemcpyDeviceToHost, s);
+  static_assert(OUT_N == 5 && ISC_N * 4 + 8 <= 1024, "pin_bytes");
+  char *pin = static_cast<char *>(h->pin);
+  const double *out = reinterpret_cast<const double *>(pin + 1024);
+  const size_t nout = size_t(OUT_N) * K;
+  cudaError_t e = cudaMemcpyAsync(pin + 1024, w->out, nout * 8, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(pin, w->isc, ISC_N * 4, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(pin + ISC_N * 4, h->H + m + int64_t(m - 1) * K, 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e);
+  res.out.assign(out, out + nout);
+  int iscv[ISC_N];
+  double hb;
+  memcpy(iscv, pin, sizeof(iscv));
+  memcpy(&hb, pin + ISC_N * 4, 8);
   if (iscv[ISC_ERR]) return iscv[ISC_ERR];
   res.m = m;
   res.r = iscv[ISC_R];

@@ -44,7 +44,8 @@ struct EigArgs {
 // Simultaneous iteration for the eigenvalues (eig_roots.cu)
 constexpr int kRootSteps32 = 14; // steps in FP32
 constexpr int kRootSteps = 20;   // and in FP64, at most; what has not converged by then goes to the QR iteration
-constexpr int kRootMinOrder = 16;  // below this order the QR iteration's few steps are as quick
+constexpr int kRootMinOrder = 6;   // below this order the QR iteration's few steps are as quick
+constexpr int kRootMin32 = 64;    // below this one an FP64 step costs little more than its launch (5 us at order 10)
 struct RootArgs {
   const double *H;    // Hessenberg matrix (ld)
   double *invsub;     // -1 / h_{i,i-1}

@@ -519,7 +519,7 @@ cudaError_t launch_roots(const RootArgs &a, int m, cudaStream_t s) {
   roots_setup_kernel<<<1, 512, 0, s>>>(a);
   if (m >= a.min_n) {
     roots_start_kernel<<<1, kRootThreads, 0, s>>>(a);
-    for (int it = 0; it < kRootSteps32; ++it) roots_step32_kernel<<<m, kRootThreads, 0, s>>>(a, it);
+    for (int it = 0; it < (m >= kRootMin32 ? kRootSteps32 : 0); ++it) roots_step32_kernel<<<m, kRootThreads, 0, s>>>(a, it);
     static_assert(kRootSteps32 % 2 == 0, "the FP64 phase starts from buffer 0");
     for (int it = 0; it < kRootSteps; ++it) roots_step_kernel<<<m, kRootThreads, 0, s>>>(a, it);
     roots_pair_kernel<<<(m + 7) / 8, 256, 0, s>>>(a);
