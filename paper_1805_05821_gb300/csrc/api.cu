@@ -42,15 +42,11 @@ bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n,
   const int base_size = basex ? s : cs;
   const int jj = (mode == PASS_FIRST) ? 0 : jcap;
   const int64_t tile_bytes = int64_t(kTile) * jj * s;
-  // FP32/BF16 passes over V: up to the register-held kernel's row pairs, unless the shared-memory form
-  // is asked for
-  const bool held = cs == 4 && g.variant == 0 && mode != PASS_FIRST && mode != PASS_FIN;
   int R = 1;
   if (jj == 0) {
     R = kMaxR;
   } else {
-    const int max_r = held ? kFusedMaxR : kMaxR;
-    while (R * 2 <= max_r && (R * 2) * tile_bytes <= g.stage_bytes) R *= 2;
+    while (R * 2 <= kMaxR && (R * 2) * tile_bytes <= g.stage_bytes) R *= 2;
   }
   // FP64 storage is bound by the FP64 pipes (2 FMAs a clock and SM): few tiles are spread over all SMs in
   // smaller stages, down to 8 KB.  (n = 4096, 11 pushes and the solve: 1.67 -> 1.30 ms.  FP32 stages
@@ -75,12 +71,7 @@ bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n,
   const bool regs = cs == 4 || (!lag && (mode == PASS_C || mode == PASS_FIRST || pass_nc_for(jcap) <= 16));
   const bool two = regs &&
                    (2 * slot_bytes + other <= g.smem_budget2) && g.max_ctas_per_sm >= 2;
-  // three where the register-held kernel has at most 16 columns a thread (and two slots fit): a stage is
-  // a chain of barriers, and the third CTA fills what is left of the other two's
-  const int G1 = kConsumers / (R * (kTile / 2));
-  const bool three = two && held && mode != PASS_A2 && R <= kFusedMaxR && (((jj + G1 - 1) / G1 + 3) & ~3) <= 16 &&
-                     2 * slot_bytes + other <= g.smem_budget3;
-  const int64_t budget = three ? g.smem_budget3 : two ? g.smem_budget2 : g.smem_budget;
+  const int64_t budget = two ? g.smem_budget2 : g.smem_budget;
   const int64_t inflight = two ? g.inflight_bytes / 2 : g.inflight_bytes;
   int slots = int((budget - other) / slot_bytes);
   const int want = int((inflight + slot_bytes - 1) / slot_bytes) + 1;
@@ -116,7 +107,7 @@ bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n,
   a.n = n;
   a.jcap = jcap;
   a.nstages = (ntiles + R - 1) / R;
-  const int per_sm = three ? 3 : two ? 2 : 1;
+  const int per_sm = two ? 2 : 1;
   grid = a.nstages < sms * per_sm ? a.nstages : sms * per_sm;
   return true;
 }

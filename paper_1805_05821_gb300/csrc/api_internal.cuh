@@ -13,7 +13,6 @@ struct Geometry {
   int64_t stage_bytes = 32 * 1024;     // target bytes of V per pipeline stage
   int64_t smem_budget = 220 * 1024;    // shared memory of a CTA when one CTA runs per SM
   int64_t smem_budget2 = 112 * 1024;   // ... when two CTAs share an SM
-  int64_t smem_budget3 = 74 * 1024;    // ... and when three do
   int64_t inflight_bytes = 96 * 1024;  // bytes of V each CTA keeps in flight
   int max_ctas_per_sm = 2;
   int variant = 0;  // FP32/BF16 passes A, B, B2: 0 = register-held stage where it fits, 1 = shared memory

@@ -18,7 +18,6 @@ constexpr int kThreads = kConsumers + 32;  // + one producer warp that issues th
 constexpr int kMaxK = 512;         // largest k_max
 constexpr int kGroup = 16;         // CTAs per first-level group of the cross-CTA reduction (see grid_reduce)
 constexpr int kMaxR = 64;          // largest number of tiles in one pipeline stage
-constexpr int kFusedMaxR = 16;     // ... of the register-held passes (one row pair a thread)
 constexpr int kMaxSlots = 8;
 
 // pass kinds (PASS_B2, PASS_A2 and PASS_FIN are the two-pass push: see lag.cuh)

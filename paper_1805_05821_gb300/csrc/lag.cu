@@ -45,7 +45,7 @@ template <typename S>
 static cudaError_t launch_lag_t(int mode, int nc, const PassArgs &a, int grid, cudaStream_t s) {
   if (mode == PASS_FIN) return launch_lag_one<S, 8, true>(a, grid, s);
   if constexpr (sizeof(typename Compute<S>::T) == 4) {
-    // FP32/BF16: the stage held in registers where it fits, else the warp-specialised kernel
+    // FP32/BF16: stages of one or two tiles held in registers, else the warp-specialised kernel
     // (row and column sweeps on different warps)
     const int fc = fused_columns(a);
     if (fc == 16) return launch_lag_fused_one<S, 16>(a, grid, s);

@@ -1,13 +1,12 @@
-// Lagged first pass of the two-pass push with the stage held in registers (FP32/BF16 storage): the
-// arithmetic of lag_ws_kernel on the thread layout of pass_fused_kernel (stages of up to 16 tiles, no
-// producer warp, two CTAs of 256 threads per SM).
+// Lagged first pass of the two-pass push with the stage held in registers (FP32/BF16 storage,
+// stages of one or two 32-row tiles): the arithmetic of lag_ws_kernel on the thread layout of
+// pass_fused_kernel (no producer warp, two CTAs of 256 threads per SM).
 //   row sweep:     per row pair, sum_c V_rc beta_pre_c and sum_c V_rc s_c over the stored columns,
 //                  from the thread's V fragment, combined across the column groups through shared
 //                  memory; the finisher of row r appends v_r = (w'_r - sum V s)/h to column jp of
 //                  V and forms w_r = (x_r - sum V beta_pre - v_r beta_pre_jp)/beta_jj;
 //   column sweep:  the stored columns' dots with w from the registers; the appended column's dot
-//                  sum_r v_r w_r accumulates in the row finishers in FP32 pairs (exact products by
-//                  fma, two-sum), which cost a stage less than FP64's 64 cycles an operation.
+//                  sum_r v_r w_r accumulates in FP64 in the row finishers.
 #pragma once
 #include "lag_ws.cuh"
 #include "pass_fused.cuh"
@@ -37,7 +36,7 @@ __global__ void __launch_bounds__(kConsumers, 2) lag_fused_kernel(const PassArgs
   double *dot = reinterpret_cast<double *>(smem + a.off_dot);
   float *combp = reinterpret_cast<float *>(smem + a.off_comb);  // row-sweep group partials, beta_pre
   float *combs = combp + 2 * kConsumers;                        //                          s
-  double *nrm = reinterpret_cast<double *>(smem + a.off_norm);  // until the norms: [warp][FC] column sums (R >= 4)
+  double *nrm = reinterpret_cast<double *>(smem + a.off_norm);
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + a.off_bar);
   volatile int *sflag = reinterpret_cast<volatile int *>(full + 2 * kMaxSlots);  // [0] abort [2] last
 
@@ -59,7 +58,6 @@ __global__ void __launch_bounds__(kConsumers, 2) lag_fused_kernel(const PassArgs
     cfs[c] = (pend && c < jt) ? static_cast<float>(a.coef2[c]) : 0.f;
   }
   for (int c = tid; c <= j; c += kConsumers) dot[c] = 0.0;
-  nrm[tid] = 0.0;
   __syncthreads();
 
   S *Vg = static_cast<S *>(const_cast<void *>(a.V));
@@ -106,28 +104,15 @@ __global__ void __launch_bounds__(kConsumers, 2) lag_fused_kernel(const PassArgs
     ncomp = (t - nsum) - y;
     nsum = t;
   };
-  // the appended column's dot, rows finished by this thread: the sum as an FP32 pair
-  float ps = 0.f, pc = 0.f;
-  auto pend_add = [&](float v, float w) {
-    const float p = __fmul_rn(v, w), pe = fmaf(v, w, -p);
-    const float t = __fadd_rn(ps, p), b = __fsub_rn(t, ps);
-    pc = __fadd_rn(pc, __fadd_rn(pe, __fadd_rn(__fsub_rn(ps, __fsub_rn(t, b)), __fsub_rn(p, b))));
-    ps = t;
-  };
+  double pacc = 0.0;  // the appended column's dot, rows finished by this thread
   auto flush = [&]() {
 #pragma unroll
     for (int u = 0; u < FC; ++u) {
       float v = cacc[u];
-      if (PF >= 32) v += __shfl_xor_sync(0xffffffffu, v, 16);
+      if (PF == 32) v += __shfl_xor_sync(0xffffffffu, v, 16);
 #pragma unroll
       for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (u < nc) {
-        if (PF <= 32) {
-          if (pr == 0) dot[c0 + u] += static_cast<double>(v);
-        } else if (lane == 0) {
-          nrm[warp * FC + u] += static_cast<double>(v);
-        }
-      }
+      if (pr == 0 && u < nc) dot[c0 + u] += static_cast<double>(v);
       cacc[u] = 0.f;
     }
   };
@@ -157,16 +142,12 @@ __global__ void __launch_bounds__(kConsumers, 2) lag_fused_kernel(const PassArgs
 #pragma unroll
       for (int u = 0; u < FC; ++u) v[u] = (has_rows && u < nc) ? ld_pair(vr + (c0 + u) * kTile) : make_float2(0.f, 0.f);
     }
-    float xv[2] = {0.f, 0.f}, wpv[2] = {0.f, 0.f};  // rows tid and tid + 256
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int rr = tid + h * kConsumers;
-      if (rr < RS) {
-        const int64_t r = r0 + rr;
-        xv[h] = xb ? float(to_c(reinterpret_cast<const S *>(sbase + a.base_off)[rr]))
-                   : ((r < a.n) ? float(to_c(xg[r])) : 0.f);
-        if (pend) wpv[h] = reinterpret_cast<const float *>(sbase + a.base2_off)[rr];
-      }
+    float xv = 0.f, wpv = 0.f;
+    if (tid < RS) {
+      const int64_t r = r0 + tid;
+      xv = xb ? float(to_c(reinterpret_cast<const S *>(sbase + a.base_off)[tid]))
+              : ((r < a.n) ? float(to_c(xg[r])) : 0.f);
+      if (pend) wpv = reinterpret_cast<const float *>(sbase + a.base2_off)[tid];
     }
     // ---------------- row sweep from registers: two coefficient vectors
     {
@@ -195,28 +176,24 @@ __global__ void __launch_bounds__(kConsumers, 2) lag_fused_kernel(const PassArgs
       const int sn = s + a.slots * gridDim.x;
       if (sn < a.nstages) issue(slot, sn);
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int rr = tid + h * kConsumers;
-      if (rr < RS) {
-        float ap = 0.f, as = 0.f;
-        for (int gg = 0; gg < G1; ++gg) {
-          ap += combp[gg * (2 * PF) + rr];
-          as += combs[gg * (2 * PF) + rr];
-        }
-        const int64_t r = r0 + rr;
-        float vn = 0.f;
-        if (pend) {
-          const S vq = Store<S>::from((wpv[h] - as) * inv_nu);
-          Vg[((r >> 5) * a.kmax + jp) * kTile + (r & 31)] = vq;
-          vn = to_c(vq);
-        }
-        const float wc = (xv[h] - (ap + vn * bp_pend)) * inv_bjj;
-        wout[r] = wc;
-        ws[rr] = wc;
-        nrm_add(xv[h] * xv[h]);
-        pend_add(vn, wc);
+    if (tid < RS) {
+      float ap = 0.f, as = 0.f;
+      for (int gg = 0; gg < G1; ++gg) {
+        ap += combp[gg * (2 * PF) + tid];
+        as += combs[gg * (2 * PF) + tid];
       }
+      const int64_t r = r0 + tid;
+      float vn = 0.f;
+      if (pend) {
+        const S vq = Store<S>::from((wpv - as) * inv_nu);
+        Vg[((r >> 5) * a.kmax + jp) * kTile + (r & 31)] = vq;
+        vn = to_c(vq);
+      }
+      const float wc = (xv - (ap + vn * bp_pend)) * inv_bjj;
+      wout[r] = wc;
+      ws[tid] = wc;
+      nrm_add(xv * xv);
+      pacc = fma(double(vn), double(wc), pacc);
     }
     named_bar_sync(1, kConsumers);  // ws complete
     // ---------------- column sweep from registers
@@ -231,20 +208,10 @@ __global__ void __launch_bounds__(kConsumers, 2) lag_fused_kernel(const PassArgs
     }
   }
   flush();
-  if (PF > 32) {  // the warps' sums of each column group, in warp order
-    named_bar_sync(1, kConsumers);
-    for (int c = tid; c < jt; c += kConsumers) {
-      const int gc = c / cpg, w0 = gc * (PF / 32);
-      double t = 0.0;
-      for (int w = w0; w < w0 + PF / 32; ++w) t += nrm[w * FC + c - gc * cpg];
-      dot[c] = t;
-    }
-    named_bar_sync(1, kConsumers);
-  }
   nrm[tid] = double(nsum) - double(ncomp);
   // the appended column's partials, one per warp (the row-sweep buffers are free after the loop)
   double *pend_part = reinterpret_cast<double *>(combp);
-  double pw = double(ps) + double(pc);
+  double pw = pacc;
 #pragma unroll
   for (int o = 16; o; o >>= 1) pw += __shfl_xor_sync(0xffffffffu, pw, o);
   if (lane == 0) pend_part[warp] = pend ? pw : 0.0;

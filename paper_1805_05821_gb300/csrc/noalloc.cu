@@ -104,7 +104,7 @@ extern "C" int foa_dmd_push_noalloc(int64_t n, int32_t k_max, int32_t dtype, voi
   h.gcount = gcount;
   h.st = st;
   h.q_host = q;
-  if (sms * 3 > kMaxGrid) return FOA_DMD_EINVAL;  // at most three CTAs per SM
+  if (sms * h.geom.max_ctas_per_sm > kMaxGrid) return FOA_DMD_EINVAL;
   // everything the kernels expect to start at zero
   cudaError_t e = cudaMemsetAsync(st, 0, kStateBytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(gcount, 0, kCountBytes, s);

@@ -228,18 +228,6 @@ __device__ __forceinline__ void pass_epilogue(const PassArgs &a, DevState *st, d
 }
 
 // ------------------------------------------------------------------------------------------
-// The order of a pass's stages: first to last, or last to first.  Each pass starts where the one before it
-// ended, with the part of V that is still in L2 (129 MB): the direction follows from the basis size, so that it is the same
-// however the push is made.  n = 1000003, j <= 100: 16.6 -> 16.3 ms for 100 pushes.
-// ------------------------------------------------------------------------------------------
-template <int MODE> __device__ __forceinline__ bool backwards(int j) {
-  if (MODE == PASS_FIRST) return false;
-  if (MODE == PASS_B2 || MODE == PASS_A2) return MODE == PASS_B2;  // two passes a push
-  return ((j + (MODE == PASS_B)) & 1) != 0;                        // three
-}
-__device__ __forceinline__ int stage_at(const PassArgs &a, int s, bool back) { return back ? a.nstages - 1 - s : s; }
-
-// ------------------------------------------------------------------------------------------
 // Filling the stage ring.  issue_v announces stage s (its V tiles and base slice) on the slot's barrier
 // and fetches the tiles; issue_base fetches the slice of x or w, when its producer has completed (a
 // partial x slice, for an unaligned x or the ragged end, is read from global memory instead).
@@ -250,10 +238,9 @@ __device__ __forceinline__ uint32_t base_bytes(const PassArgs &a, int t0, int nt
   return bulk ? uint32_t(nt) * kTile * sizeof(BaseT) : 0u;
 }
 template <typename S, typename BaseT, bool kBaseX>
-__device__ __forceinline__ void issue_v(const PassArgs &a, int j, int slot, int s, bool back, unsigned char *slots,
-                                        uint64_t *full) {
+__device__ __forceinline__ void issue_v(const PassArgs &a, int j, int slot, int s, unsigned char *slots, uint64_t *full) {
   if (s >= a.nstages) return;
-  const int t0 = stage_at(a, s, back) * a.R, nt = min(a.R, a.ntiles - t0);
+  const int t0 = s * a.R, nt = min(a.R, a.ntiles - t0);
   const uint32_t tile_bytes = uint32_t(kTile) * uint32_t(j) * sizeof(S);
   unsigned char *dst = slots + size_t(slot) * a.slot_bytes;
   mbar_arrive_expect_tx(&full[slot], uint32_t(nt) * tile_bytes + base_bytes<BaseT, kBaseX>(a, t0, nt));
@@ -263,10 +250,10 @@ __device__ __forceinline__ void issue_v(const PassArgs &a, int j, int slot, int 
                &full[slot]);
 }
 template <typename BaseT, bool kBaseX>
-__device__ __forceinline__ void issue_base(const PassArgs &a, const BaseT *bg, int slot, int s, bool back,
-                                           unsigned char *slots, uint64_t *full) {
+__device__ __forceinline__ void issue_base(const PassArgs &a, const BaseT *bg, int slot, int s, unsigned char *slots,
+                                           uint64_t *full) {
   if (s >= a.nstages) return;
-  const int t0 = stage_at(a, s, back) * a.R, nt = min(a.R, a.ntiles - t0);
+  const int t0 = s * a.R, nt = min(a.R, a.ntiles - t0);
   const uint32_t bytes = base_bytes<BaseT, kBaseX>(a, t0, nt);
   if (bytes) bulk_g2s(slots + size_t(slot) * a.slot_bytes + a.base_off, bg + int64_t(t0) * kTile, bytes, &full[slot]);
 }
@@ -335,18 +322,16 @@ __global__ void __launch_bounds__(kThreads, pass_min_blocks<S, NC>()) pass_kerne
   // the ring's first stages of V before the predecessor is waited for, their base slices after it
   const int jp = prefetch_columns<MODE>(a, st);
   if (tid == kIssuer && jp)
-    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, backwards<MODE>(jp), slots, full);
+    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, slots, full);
   pdl_wait();
   pdl_trigger();
   if (tid == kIssuer && jp)
-    for (int k = 0; k < a.slots; ++k)
-      issue_base<BaseT, kBaseX>(a, baseg, k, blockIdx.x + k * gridDim.x, backwards<MODE>(jp), slots, full);
+    for (int k = 0; k < a.slots; ++k) issue_base<BaseT, kBaseX>(a, baseg, k, blockIdx.x + k * gridDim.x, slots, full);
   const int j = (MODE == PASS_FIRST) ? 0 : st->j;
   if (!st->active || (MODE == PASS_FIRST ? st->j != 0 : (j < 1 || j > a.jcap)) || (jp && jp != j)) {
     if (tid == kIssuer && jp) drain(a, full);
     return;
   }
-  const bool back = backwards<MODE>(j);
   // QR view (a.form): pass A projects x itself (w = x, no pre-vector)
   const bool qr_a = (MODE == PASS_A) && a.form != 0;
   const double cscale = (MODE == PASS_A && !qr_a) ? st->inv_bjj : 1.0;
@@ -368,8 +353,8 @@ __global__ void __launch_bounds__(kThreads, pass_min_blocks<S, NC>()) pass_kerne
           break;
         }
         if (sflag[0]) break;
-        issue_v<S, BaseT, kBaseX>(a, j, slot, s, back, slots, full);
-        issue_base<BaseT, kBaseX>(a, baseg, slot, s, back, slots, full);
+        issue_v<S, BaseT, kBaseX>(a, j, slot, s, slots, full);
+        issue_base<BaseT, kBaseX>(a, baseg, slot, s, slots, full);
       }
     }
     return;
@@ -432,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, pass_min_blocks<S, NC>()) pass_kerne
       atomicExch(&st->err, FOA_DMD_ETIMEOUT);
     }
     C *ws = wsb + (it & 1) * (a.R * kTile);  // double buffer: the next row sweep may start early
-    const int t0 = stage_at(a, s, back) * a.R;
+    const int t0 = s * a.R;
     const int nt = min(a.R, a.ntiles - t0);
     const int RS = nt * kTile;
     const int64_t r0 = int64_t(t0) * kTile;

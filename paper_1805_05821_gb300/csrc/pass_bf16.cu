@@ -60,21 +60,12 @@ static cudaError_t launch_dots(int nc, const PassArgs &a, int grid, cudaStream_t
   }
 }
 
-// pass C: the register-held kernel where its column groups fit
-static cudaError_t launch_c(const PassArgs &a, int grid, cudaStream_t s) {
-  const int fc = fused_columns(a);
-  if (fc == 16) return launch_fused_one<PASS_C, 16>(a, grid, s);
-  if (fc == 24) return launch_fused_one<PASS_C, 24>(a, grid, s);
-  if (fc == 32) return launch_fused_one<PASS_C, 32>(a, grid, s);
-  return launch_one<PASS_C, 8>(a, grid, s);
-}
-
 cudaError_t launch_pass_bf16(int mode, int nc, const PassArgs &a, int grid, cudaStream_t s) {
   switch (mode) {
     case PASS_A: return launch_dots<PASS_A>(nc, a, grid, s);
     case PASS_B: return launch_dots<PASS_B>(nc, a, grid, s);
     case PASS_B2: return launch_dots<PASS_B2>(nc, a, grid, s);
-    case PASS_C: return launch_c(a, grid, s);
+    case PASS_C: return launch_one<PASS_C, 8>(a, grid, s);
     default: return launch_one<PASS_FIRST, 8>(a, grid, s);
   }
 }

@@ -63,18 +63,16 @@ __global__ void __launch_bounds__(kThreads, 2) pass_ws_kernel(const PassArgs a) 
   // the ring's first stages of V before the predecessor is waited for, their base slices after it
   const int jp = prefetch_columns<MODE>(a, st);
   if (tid == kIssuer && jp)
-    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, backwards<MODE>(jp), slots, full);
+    for (int k = 0; k < a.slots; ++k) issue_v<S, BaseT, kBaseX>(a, jp, k, blockIdx.x + k * gridDim.x, slots, full);
   pdl_wait();
   pdl_trigger();
   if (tid == kIssuer && jp)
-    for (int k = 0; k < a.slots; ++k)
-      issue_base<BaseT, kBaseX>(a, baseg, k, blockIdx.x + k * gridDim.x, backwards<MODE>(jp), slots, full);
+    for (int k = 0; k < a.slots; ++k) issue_base<BaseT, kBaseX>(a, baseg, k, blockIdx.x + k * gridDim.x, slots, full);
   const int j = st->j;
   if (!st->active || j < 1 || j > a.jcap || (jp && jp != j)) {
     if (tid == kIssuer && jp) drain(a, full);
     return;
   }
-  const bool back = backwards<MODE>(j);
   // QR view (a.form): pass A projects x itself (w = x, no pre-vector)
   const bool qr_a = (MODE == PASS_A) && a.form != 0;
   const float cscale = (MODE == PASS_A && !qr_a) ? float(st->inv_bjj) : 1.f;
@@ -96,8 +94,8 @@ __global__ void __launch_bounds__(kThreads, 2) pass_ws_kernel(const PassArgs a) 
           break;
         }
         if (sflag[0]) break;
-        issue_v<S, BaseT, kBaseX>(a, j, slot, s, back, slots, full);
-        issue_base<BaseT, kBaseX>(a, baseg, slot, s, back, slots, full);
+        issue_v<S, BaseT, kBaseX>(a, j, slot, s, slots, full);
+        issue_base<BaseT, kBaseX>(a, baseg, slot, s, slots, full);
       }
     }
     return;
@@ -128,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, 2) pass_ws_kernel(const PassArgs a) 
       }
       float *ws = wsb + b * (a.R * kTile);
       float *cb = combb + b * 256;
-      const int t0 = stage_at(a, s, back) * a.R;
+      const int t0 = s * a.R;
       const int nt = min(a.R, a.ntiles - t0);
       const int RS = nt * kTile;
       const int64_t r0 = int64_t(t0) * kTile;
@@ -249,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, 2) pass_ws_kernel(const PassArgs a) 
         atomicExch(&st->err, FOA_DMD_ETIMEOUT);
       }
       const float *ws = wsb + b * (a.R * kTile);
-      const int t0 = stage_at(a, s, back) * a.R;
+      const int t0 = s * a.R;
       const int nt = min(a.R, a.ntiles - t0);
       const S *vs = reinterpret_cast<const S *>(slots + size_t(slot) * a.slot_bytes);
       for (int kt = 0; kt < nt; ++kt) {

@@ -1,0 +1,64 @@
+"""The order in which a push adds in FP32 is part of its result: a Ritz vector's amplitude magnifies a change of
+H-bar by the eigenvectors' condition (11 to 89 for the 2-D waves), so a different order of the same sums
+moves it by up to 2e-5.  The values of golden/push_order.json are those of the documented order (the stages
+of a pass first to last, two CTAs per SM; row sums and column dots as in pass_ws.cuh, pass_fused.cuh, pass.cuh and lag*.cuh) on
+a GB300's 152 SMs, for inputs that are the same on every machine.  The basis is compared bit for bit (a sum
+of the bit patterns of every column), H-bar's subdiagonal and beta's last column to 1e-12, which
+leaves room for the order of the FP64 sums."""
+import json
+import os
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "push_order.json")
+#            dtype, n, N, reorth, form: stages of 16 tiles and more down to one, several stages a CTA
+CASES = {"f32": ("f32", 400001, 140, 1, 0), "bf16": ("bf16", 400001, 150, 1, 0),
+         "f32_qr": ("f32", 100003, 70, 1, 1), "f32_cgs1": ("f32", 100003, 70, 0, 0),
+         "f32_two_pass": ("f32", 400001, 140, 2, 0), "bf16_two_pass": ("bf16", 100003, 70, 2, 0)}
+
+
+def snapshot_rows(n, N):
+    """x_0 noise, x_t = 7/8 x_{t-1} + noise, in FP32: integer arithmetic and separately rounded operations."""
+    i = np.arange(n, dtype=np.uint64)
+    x = np.zeros(n, dtype=np.float32)
+    for t in range(N):
+        k = (i + np.uint64(t * n + 1)) * np.uint64(6364136223846793005)
+        k ^= k >> np.uint64(29)
+        k *= np.uint64(0xBF58476D1CE4E5B9)
+        x = x * np.float32(0.875) + ((k >> np.uint64(48)).astype(np.float32) - np.float32(32767.5)) * np.float32(2.0 ** -16)
+        yield x
+
+
+def record(F, dt, n, N, reorth, form):
+    import torch
+    g = F.FoaDMD(n, N, dt, reorth=reorth, form=form)
+    td = {"f32": torch.float32, "bf16": torch.bfloat16}[dt]
+    for x in snapshot_rows(n, N):
+        st, info = g.push(torch.from_numpy(x).cuda().to(td))
+        assert st == 0, info
+    q, _, H, B = g.state()
+    assert q == N
+    V = g.basis(0, N).contiguous()
+    bits = V.view(torch.int32 if dt == "f32" else torch.int16).to(torch.int64).sum(dim=1).cpu().tolist()
+    sub = [float(H[c + 1, c]) for c in range(N - 1)]
+    g.close()
+    return {"bits": bits, "sub": sub, "last": [float(v) for v in B[:N, N - 1]]}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_order_of_the_sums(name):
+    import torch
+    from paper_1805_05821_gb300 import build, foa_dmd
+    build.build()
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the stages are dealt over 152 SMs")
+    want = json.load(open(GOLDEN))[name]
+    got = record(foa_dmd, *CASES[name])
+    bad = [c for c in range(len(want["bits"])) if want["bits"][c] != got["bits"][c]]
+    for key in ("sub", "last"):
+        w, g = np.array(want[key]), np.array(got[key])
+        assert np.abs(g - w).max() <= 1e-12 * np.abs(w).max(), (key, np.abs(g - w).max())
+    assert not bad, f"columns {bad[:8]} of {len(want['bits'])} differ in their bits"
