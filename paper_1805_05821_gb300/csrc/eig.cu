@@ -494,8 +494,8 @@ __global__ void order_kernel(EigArgs e, int nsel) {
     e.perm[p] = i;
   }
   __syncthreads();
-  // sorted y columns 0..nsel-1
-  for (int64_t t = threadIdx.x; t < int64_t(nsel) * m; t += blockDim.x) {
+  // sorted y columns 0..min(nsel, r)-1 (perm has r entries)
+  for (int64_t t = threadIdx.x; t < int64_t(min(nsel, r)) * m; t += blockDim.x) {
     const int c = int(t / m), i = int(t % m);
     const int src = e.perm[c];
     e.ysr[i + int64_t(c) * e.ld] = e.yr[i + int64_t(src) * e.ld];
