@@ -210,6 +210,13 @@ int foa_dmd_eig(foa_dmd_t *h, double rank_tol, foa_dmd_eig_result *res);
 int foa_dmd_test_wait_fault(foa_dmd_t *h, int32_t skip_cta, int64_t spin_cycles);
 
 /*
+ * Test hook: how the last foa_dmd_eig of this handle found its eigenvalues.  *qr: 1 if the QR iteration
+ * did, 0 if the simultaneous iteration's values stood; *steps: the FP64 steps of the
+ * simultaneous iteration that converged (0 where it did not run or not converge).  Errors: EINVAL.
+ */
+int foa_dmd_test_eig_path(foa_dmd_t *h, int32_t *qr, int32_t *steps);
+
+/*
  * Copy the FP64 state to host buffers (synchronises): q, stopped flag, H-bar and beta as
  * k_max x k_max column-major arrays with leading dimension ld >= k_max (either may be NULL).
  */

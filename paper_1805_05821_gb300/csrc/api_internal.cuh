@@ -77,6 +77,7 @@ struct foa_dmd {
   // foa_dmd_test_wait_fault: one-shot failure injection into the next cooperative SVD launch
   int test_skip_cta = -1;
   long long test_spin_cycles = 0;
+  int32_t eig_path[2] = {0, 0};  // of the last foa_dmd_eig: QR iteration ran, FP64 steps (foa_dmd_test_eig_path)
 };
 
 namespace foa {

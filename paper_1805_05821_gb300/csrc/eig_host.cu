@@ -246,6 +246,8 @@ static int run_eig_body(foa_dmd *h, double rank_tol, int nsel, EigOut &res) {
   double hb;
   memcpy(iscv, pin, sizeof(iscv));
   memcpy(&hb, pin + ISC_N * 4, 8);
+  h->eig_path[0] = iscv[ISC_QR] != 0;
+  h->eig_path[1] = iscv[ISC_ITS];
   if (iscv[ISC_ERR]) return iscv[ISC_ERR];
   res.m = m;
   res.r = iscv[ISC_R];
@@ -338,6 +340,13 @@ extern "C" int foa_dmd_test_wait_fault(foa_dmd_t *h, int32_t skip_cta, int64_t s
   if (!h || skip_cta < 0 || spin_cycles < 1 || spin_cycles > kGridSpinCycles) return FOA_DMD_EINVAL;
   h->test_skip_cta = skip_cta;
   h->test_spin_cycles = spin_cycles;
+  return FOA_DMD_OK;
+}
+
+extern "C" int foa_dmd_test_eig_path(foa_dmd_t *h, int32_t *qr, int32_t *steps) {
+  if (!h || !qr || !steps) return FOA_DMD_EINVAL;
+  *qr = h->eig_path[0];
+  *steps = h->eig_path[1];
   return FOA_DMD_OK;
 }
 

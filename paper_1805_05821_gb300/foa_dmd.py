@@ -77,6 +77,7 @@ def lib():
                                                   ctypes.POINTER(i32)]),
             "foa_dmd_eig": (ctypes.c_int, [vp, d, ctypes.POINTER(foa_dmd_eig_result)]),
             "foa_dmd_test_wait_fault": (ctypes.c_int, [vp, i32, i64]),
+            "foa_dmd_test_eig_path": (ctypes.c_int, [vp, ctypes.POINTER(i32), ctypes.POINTER(i32)]),
             "foa_dmd_check_status": (ctypes.c_int, [ctypes.POINTER(ctypes.c_uint32)]),
             "foa_dmd_get_state": (ctypes.c_int, [vp, ctypes.POINTER(i32), ctypes.POINTER(i32), _DP, _DP, i32]),
             "foa_dmd_get_basis": (ctypes.c_int, [vp, i32, i32, vp, i64]),
@@ -243,6 +244,13 @@ def foa_dmd_check_status():
 
 def foa_dmd_test_wait_fault(h, skip_cta, spin_cycles):
     return lib().foa_dmd_test_wait_fault(h, int(skip_cta), int(spin_cycles))
+
+
+def foa_dmd_test_eig_path(h):
+    """(QR iteration ran, FP64 steps of the simultaneous iteration) of the last eig."""
+    qr, steps = ctypes.c_int32(0), ctypes.c_int32(0)
+    _check(lib().foa_dmd_test_eig_path(h, ctypes.byref(qr), ctypes.byref(steps)), "foa_dmd_test_eig_path")
+    return bool(qr.value), steps.value
 
 
 def foa_dmd_push_noalloc(n, k_max, dtype, V, Hbar, beta, q, x, w, breakdown_tol=0.0, stream=None):

@@ -38,3 +38,20 @@ def test_more_columns_asked_for_than_the_rank(m, r, tmp_path):
         assert a[key].shape == b[key].shape and np.array_equal(a[key], b[key]), key
     g.close()
     h.close()
+
+
+@pytest.mark.parametrize("kind,m", [("waves", m) for m in (1, 5, 6, 16, 17, 33, 63, 64, 65, 129, 256, 383, 511)]
+                         + [("multiple", 50), ("split", 40), ("scaled", 40)])
+def test_which_iteration_found_the_eigenvalues(kind, m, tmp_path):
+    """Near-orthogonal matrices of order 6 and more are solved by the simultaneous iteration within
+    its 20 FP64 steps; repeated eigenvalues, a zero subdiagonal and entries far outside FP32's range
+    are left to the QR iteration."""
+    from paper_1805_05821_gb300.foa_dmd import foa_dmd_test_eig_path
+    g = load_with(matrix(kind, m, 7 * m + len(kind)), tmp_path / "h.ckpt")
+    assert g.eig(0.0)["status"] == 0
+    qr, steps = foa_dmd_test_eig_path(g.h)
+    if kind == "waves":
+        assert qr == (m < 6) and (m < 6 or 0 < steps <= 20), (qr, steps)
+    else:
+        assert qr
+    g.close()
