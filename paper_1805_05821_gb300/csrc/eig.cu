@@ -155,7 +155,7 @@ __global__ void hessenberg_kernel(double *G, int ldg, double *Q, int ldq, const 
 __global__ void hqr_kernel(double *Ag, int lda, const int *isc_in, double *wr, double *wi, int *isc,
                            int smem_elems) {
   const int n = isc_in[ISC_R];
-  if (!isc_in[ISC_QR]) return;
+  if (!isc_in[ISC_QR] && !isc_in[ISC_RES]) return;
   extern __shared__ double sh[];
   const int tid = threadIdx.x, lane = tid & 31;
   const int T1 = blockDim.x - 32;  // threads outside warp 0

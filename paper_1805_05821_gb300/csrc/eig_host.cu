@@ -54,7 +54,7 @@ static int eig_alloc(foa_dmd *h, EigWork **slot) {
   } while (0)
   AL(w->A, 2 * K2); AL(w->U, K2); AL(w->sig_raw, K1); AL(w->sig, K1); AL(w->G, K2); AL(w->Q, K2); AL(w->T, 2 * K2);
   AL(w->Aqr, K2); AL(w->wr, K1); AL(w->wi, K1); AL(w->yr, K2); AL(w->yi, K2); AL(w->ysr, K2); AL(w->ysi, K2);
-  AL(w->ind, K1); AL(w->amp_re, K1); AL(w->amp_im, K1); AL(w->out, OUT_N * K1); AL(w->rscal, 5 * 8);
+  AL(w->ind, K1); AL(w->amp_re, K1); AL(w->amp_im, K1); AL(w->out, OUT_N * K1); AL(w->rscal, 6 * 8);
   AL(w->vec, 4 * K2); AL(w->invsub, K1); AL(w->zr, 2 * K1); AL(w->zi, 2 * K1); AL(w->dold, K1);
   AL(w->conv, size_t(K) * 4); AL(w->part, size_t(K) * 4); AL(w->hf, (size_t(K) + 1) * K * 4); AL(w->left, kRootSteps * 4);
   AL(w->tw, size_t(w->vgrid) * 2 * K1); AL(w->yplanes, 2 * K2);
@@ -151,22 +151,6 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   ra.min_n = kRootMinOrder;
   e = launch_roots(ra, m, s);
   if (e != cudaSuccess) return cuda_status(e);
-  e = cudaMemcpyAsync(w->Aqr, w->G, size_t(K) * K * 8, cudaMemcpyDeviceToDevice, s);
-  if (e != cudaSuccess) return cuda_status(e);
-  // The QR iteration runs where the simultaneous iteration does not apply or has not converged
-  // (isc[ISC_QR]).  It works on the r x r matrix (r = m without truncation); r is counted on the
-  // device.  The launch offers the band |j - i| <= 3 (7 m doubles) and up to 160^2 doubles for the
-  // whole matrix, which the kernel copies to shared memory when r^2 fits (every truncated eig with
-  // r <= 160, whatever m).
-  const size_t band = 7 * size_t(m);
-  const size_t full = std::min(std::min(size_t(m) * m, size_t(kQrSmemMaxOrder) * kQrSmemMaxOrder),
-                               size_t(232448 / 8) - band - 512);  // 4 KB left for the static variables
-  const size_t qr_smem = (full + band) * 8;
-  if (qr_smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(hqr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(qr_smem));
-    if (e != cudaSuccess) return cuda_status(e);
-  }
-  hqr_kernel<<<1, 512, qr_smem, s>>>(w->Aqr, K, w->isc, w->wr, w->wi, w->isc, int(full));
   EigArgs a;
   memset(&a, 0, sizeof(a));
   a.Hs = w->G;
@@ -196,12 +180,34 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   a.have_u = trunc ? 1 : 0;
   a.hlast_p = trunc ? h->H + m + int64_t(m - 1) * K : w->scal;  // h_{m+1,m} (0 after a breakdown)
   a.b11_p = trunc ? h->B : w->scal + 1;
+  if (m >= kRootMinOrder) {
+    e = launch_invit(a, false, s);
+    if (e != cudaSuccess) return cuda_status(e);
+  }
+  e = cudaMemcpyAsync(w->Aqr, w->G, size_t(K) * K * 8, cudaMemcpyDeviceToDevice, s);
+  if (e != cudaSuccess) return cuda_status(e);
+  // The QR iteration runs where the simultaneous iteration does not apply or has not converged
+  // (isc[ISC_QR]), or where the inverse iteration did not confirm a value (isc[ISC_RES]).  It works
+  // on the r x r matrix (r = m without truncation); r is counted on the device.  The launch offers the
+  // band |j - i| <= 3 (7 m doubles) and up to 160^2 doubles for the whole matrix, which the kernel
+  // copies to shared memory when r^2 fits (every truncated eig with r <= 160, whatever m).
+  const size_t band = 7 * size_t(m);
+  const size_t full = std::min(std::min(size_t(m) * m, size_t(kQrSmemMaxOrder) * kQrSmemMaxOrder),
+                               size_t(232448 / 8) - band - 512);  // 4 KB left for the static variables
+  const size_t qr_smem = (full + band) * 8;
+  if (qr_smem > 48 * 1024) {
+    e = cudaFuncSetAttribute(hqr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(qr_smem));
+    if (e != cudaSuccess) return cuda_status(e);
+  }
+  hqr_kernel<<<1, 512, qr_smem, s>>>(w->Aqr, K, w->isc, w->wr, w->wi, w->isc, int(full));
+  e = launch_invit(a, true, s);
+  if (e != cudaSuccess) return cuda_status(e);
   e = launch_vectors(a, w->vgrid, s);
   if (e != cudaSuccess) return cuda_status(e);
   if (nsel > m) nsel = m;
   order_kernel<<<1, 512, size_t(m) * 20 + 64, s>>>(a, nsel);
-  // roots_setup (start, steps, pair, finish), hqr, flip, invit, vectors, order
-  h->launches += 6 + (m >= kRootMin32 ? kRootSteps32 : 0) + (m >= kRootMinOrder ? kRootSteps + 3 : 0);
+  // roots_setup (start, steps, pair, finish, flip, invit), hqr, flip, invit, vectors, order
+  h->launches += 6 + (m >= kRootMin32 ? kRootSteps32 : 0) + (m >= kRootMinOrder ? kRootSteps + 5 : 0);
   if (trunc && copied) {
     e = cudaEventRecord(copied, s);
     if (e != cudaSuccess) return cuda_status(e);
@@ -246,7 +252,7 @@ static int run_eig_body(foa_dmd *h, double rank_tol, int nsel, EigOut &res) {
   double hb;
   memcpy(iscv, pin, sizeof(iscv));
   memcpy(&hb, pin + ISC_N * 4, 8);
-  h->eig_path[0] = iscv[ISC_QR] != 0;
+  h->eig_path[0] = iscv[ISC_QR] || iscv[ISC_RES];
   h->eig_path[1] = iscv[ISC_ITS];
   if (iscv[ISC_ERR]) return iscv[ISC_ERR];
   res.m = m;

@@ -14,7 +14,8 @@ struct GridBar {
 };
 
 // integer scalars of one eigen-decomposition (device)
-enum { ISC_R = 0, ISC_STATUS = 1, ISC_ERR = 2, ISC_ROT = 3, ISC_SWEEPS = 4, ISC_QR = 5, ISC_ITS = 6, ISC_N = 16 };
+enum { ISC_R = 0, ISC_STATUS = 1, ISC_ERR = 2, ISC_ROT = 3, ISC_SWEEPS = 4, ISC_QR = 5, ISC_ITS = 6, ISC_RES = 7,
+       ISC_N = 16 };  // QR: no values from the simultaneous iteration; RES: values that invit_kernel did not confirm
 // rows of the sorted output block (each ld long)
 enum { OUT_LRE = 0, OUT_LIM = 1, OUT_IND = 2, OUT_ARE = 3, OUT_AIM = 4, OUT_N = 5 };
 
@@ -25,7 +26,7 @@ struct EigArgs {
   const double *H;    // H-bar of the stream (ldH), for the truncated indicator
   int ldH;
   const double *wr, *wi;
-  const double *anorm;
+  const double *anorm;  // roots_setup_kernel's scal
   double *M;          // Hs transposed and flipped about its antidiagonal (r x r, ld)
   double *vec;        // inverse iteration: Re z, Im z, Re w, Im w planes of ld x ld (eigenvectors of Hs)
   double *tw;         // per-CTA scratch
@@ -60,6 +61,7 @@ struct RootArgs {
   int ld, min_n;
 };
 cudaError_t launch_roots(const RootArgs &a, int m, cudaStream_t s);
+cudaError_t launch_invit(const EigArgs &e, bool after_qr, cudaStream_t s);
 cudaError_t launch_vectors(const EigArgs &e, int vgrid, cudaStream_t s);
 
 // one push-time indicator (device ring written by the indicator stream)

@@ -218,7 +218,8 @@ __device__ __forceinline__ int hyman_any(const T *H, int ld, int n, const T *inv
 }
 
 // One CTA.  scal: [0] sum |h_ij| over the Hessenberg part (also the pivot floor of the inverse
-// iteration), [1] tr H, [2] tr H^2, [3] ||H - tr(H)/n||_F / sqrt(n), [4] log2 of the subdiagonals' product.
+// iteration), [1] tr H, [2] tr H^2, [3] ||H - tr(H)/n||_F / sqrt(n), [4] log2 of the subdiagonals' product,
+// [5] ||H||_F.
 __global__ void __launch_bounds__(512) roots_setup_kernel(RootArgs a) {
   const int n = a.isc[ISC_R];
   const int tid = threadIdx.x;
@@ -275,6 +276,7 @@ __global__ void __launch_bounds__(512) roots_setup_kernel(RootArgs a) {
     a.scal[2] = t2;
     a.scal[3] = fro;
     a.scal[4] = ls;
+    a.scal[5] = sqrt(fr);
     a.isc[ISC_QR] = bad;
   }
 }
@@ -424,18 +426,19 @@ __global__ void __launch_bounds__(kRootThreads) roots_step_kernel(RootArgs a, in
   }
 }
 
-// For each value the one nearest to its conjugate: a warp per value
+// For each value the one nearest to its conjugate, and its nearest neighbour: a warp per value
 __global__ void __launch_bounds__(256) roots_pair_kernel(RootArgs a) {
   const int n = a.isc[ISC_R], i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (a.isc[ISC_QR] || i >= n) return;
   const int last = last_step(a);
   if (last < 0) return;
   const double *zr = a.zr + ((last & 1) ^ 1) * a.ld, *zi = a.zi + ((last & 1) ^ 1) * a.ld;
-  double best = 1e300;
+  double best = 1e300, near = 1e300;
   int arg = i;
   for (int j = lane; j < n; j += 32) {
-    const double dr = zr[j] - zr[i], di = zi[j] + zi[i];
+    const double dr = zr[j] - zr[i], di = zi[j] + zi[i], ds = zi[j] - zi[i];
     const double d = fma(dr, dr, di * di);
+    if (j != i) near = fmin(near, fma(dr, dr, ds * ds));
     if (d < best) {
       best = d;
       arg = j;
@@ -450,13 +453,17 @@ __global__ void __launch_bounds__(256) roots_pair_kernel(RootArgs a) {
       arg = oa;
     }
   }
+  // two values this close may be one eigenvalue found twice
+  if (!(near > 1e-18 * a.scal[3] * a.scal[3])) a.isc[ISC_QR] = 1;
   if (lane == 0) a.part[i] = arg;
 }
 
 // Pair the values, check them, and store them as the QR iteration does (a conjugate pair side by
-// side, +Im first).  They stand if all converged, each value's nearest conjugate has that value as
-// its own nearest one (a real eigenvalue is its own), and both traces agree: a value found twice in
-// place of another one would change them.  Otherwise isc[ISC_QR] asks for the QR iteration.
+// side, +Im first).  They are passed on if all converged, no two are within 1e-9 of the spectrum's size,
+// each value's nearest conjugate has that value as its own nearest one (a real eigenvalue is its
+// own), and both traces agree: a value found twice in place of another one would change them.  Otherwise
+// isc[ISC_QR] asks for the QR iteration.  Whether each is as accurate as the QR iteration's decides the
+// inverse iteration (invit_kernel), which takes the pairs' means as they are stored here.
 __global__ void __launch_bounds__(512) roots_finish_kernel(RootArgs a) {
   const int n = a.isc[ISC_R], tid = threadIdx.x, K = a.ld;
   if (a.isc[ISC_QR]) return;

@@ -55,3 +55,56 @@ def test_which_iteration_found_the_eigenvalues(kind, m, tmp_path):
     else:
         assert qr
     g.close()
+
+
+def hard_matrix(kind, m, seed):
+    """Hessenberg matrices whose eigenvalues the simultaneous iteration approaches slowly or at different scales."""
+    import scipy.linalg as sl
+    g = np.random.default_rng(seed)
+    Q = np.linalg.qr(g.standard_normal((m, m)))[0]
+    name, val = kind.split(":")
+    val = float(val)
+    A = np.zeros((m, m))
+    ang = np.sort(g.uniform(0.2, 2.9, m // 2))
+    if name.startswith("group"):  # one group of 2 or 3 angles, val apart
+        c, o = int(name[5:]), m // 6
+        ang[o:o + c] = ang[o] + val * np.arange(c)
+    if name == "cluster":  # groups of six conjugate pairs on the unit circle, val apart
+        ang = np.repeat(ang[::6], 6)[:m // 2] + val * np.tile(np.arange(6), m // 12 + 1)[:m // 2]
+    rad = np.ones(m // 2)
+    if name == "graded":  # moduli from 1 to 10^-val
+        rad = 10.0 ** (-val * np.linspace(0, 1, m // 2))
+    for k in range(m // 2):
+        c, s = rad[k] * np.cos(ang[k]), rad[k] * np.sin(ang[k])
+        A[2 * k:2 * k + 2, 2 * k:2 * k + 2] = [[c, -s], [s, c]]
+    if name == "nonnormal":  # far from normal: entries up to val above the diagonal blocks
+        A += val * np.triu(g.standard_normal((m, m)), 2) / m
+    return np.triu(sl.hessenberg(Q @ A @ Q.T), -1)
+
+
+@pytest.mark.parametrize("m", [40, 96, 130])
+@pytest.mark.parametrize("kind", ["group2:1e-6", "group2:1e-7", "group2:1e-8", "group2:1e-9", "group2:1e-10", "group3:1e-6",
+                                  "group3:1e-7", "cluster:1e-4", "cluster:1e-7", "graded:6", "graded:10",
+                                  "nonnormal:10", "nonnormal:1000"])
+def test_eigenvalues_are_backward_stable(kind, m, tmp_path):
+    """Whichever iteration found them, each eigenvalue is one of a matrix within 32 m eps ||H||_F of H: the
+    smallest singular value of H - lambda says so directly.  And all are there: matched with LAPACK's,
+    they differ by at most that over s_i."""
+    import scipy.linalg as sl
+    import scipy.optimize as so
+    H = hard_matrix(kind, m, m + len(kind))
+    g = load_with(H, tmp_path / "h.ckpt")
+    res = g.eig(0.0)
+    assert res["status"] == 0
+    nrm = np.linalg.norm(H)
+    back = np.array([np.linalg.svd(H - x * np.eye(m), compute_uv=False)[-1] for x in res["lam"]])
+    lam, L, R = sl.eig(H, left=True, right=True)
+    s = np.abs(np.sum(L.conj() * R, 0))
+    d = np.abs(res["lam"][:, None] - lam[None, :])
+    i, j = so.linear_sum_assignment(d)
+    from paper_1805_05821_gb300.foa_dmd import foa_dmd_test_eig_path
+    print(kind, m, "path", foa_dmd_test_eig_path(g.h), "backward error / (m eps |H|) %.3g" % (back.max() / (m * EPS * nrm)),
+          "forward / (m eps |H| / s) %.3g" % (d[i, j] * s[j]).max().__truediv__(m * EPS * nrm), "s %.1e" % s.min())
+    g.close()
+    assert back.max() <= 32 * m * EPS * nrm
+    assert (d[i, j] * s[j]).max() <= 64 * m * EPS * nrm  # LAPACK's own error added
