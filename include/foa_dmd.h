@@ -211,8 +211,8 @@ int foa_dmd_test_wait_fault(foa_dmd_t *h, int32_t skip_cta, int64_t spin_cycles)
 
 /*
  * Test hook: how the last foa_dmd_eig of this handle found its eigenvalues.  *qr: 1 if the QR iteration
- * did, 0 if the simultaneous iteration's values stood; *steps: the FP64 steps of the
- * simultaneous iteration that converged (0 where it did not run or not converge).  Errors: EINVAL.
+ * did, 0 if the simultaneous iteration's values stood; *steps: the FP64 steps that the simultaneous
+ * iteration took (0 where it does not apply).  Errors: EINVAL.
  */
 int foa_dmd_test_eig_path(foa_dmd_t *h, int32_t *qr, int32_t *steps);
 

@@ -57,6 +57,22 @@ def test_which_iteration_found_the_eigenvalues(kind, m, tmp_path):
     g.close()
 
 
+@pytest.mark.parametrize("m,e", [(128, -160), (40, -160), (128, 160), (128, -100), (128, 40), (128, -40)])
+def test_scale_decides_without_a_step(m, e, tmp_path):
+    """Entries whose scale FP32 cannot hold go to the QR iteration before any step is tried; 2^+-40 does not."""
+    from paper_1805_05821_gb300.foa_dmd import foa_dmd_test_eig_path
+    H = matrix("waves", m, m)
+    g = load_with(np.ldexp(H, e), tmp_path / "h.ckpt")
+    res = g.eig(0.0)
+    qr, steps = foa_dmd_test_eig_path(g.h)
+    assert res["status"] == 0
+    assert (qr, steps) == (True, 0) if abs(e) > 60 else (not qr and steps > 0), (qr, steps)
+    lam = np.linalg.eigvals(H)
+    d = np.abs(np.ldexp(res["lam"].real, -e)[:, None] + 1j * np.ldexp(res["lam"].imag, -e)[:, None] - lam[None, :])
+    assert d.min(axis=1).max() <= 64 * m * EPS * np.linalg.norm(H)  # normal to 1e-3: s_i near 1
+    g.close()
+
+
 def hard_matrix(kind, m, seed):
     """Hessenberg matrices whose eigenvalues the simultaneous iteration approaches slowly or at different scales."""
     import scipy.linalg as sl
