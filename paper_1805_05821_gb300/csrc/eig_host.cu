@@ -149,7 +149,7 @@ static int enqueue_eig(foa_dmd *h, EigWork *w, cudaStream_t s, int m, double ran
   ra.isc = w->isc;
   ra.ld = K;
   ra.min_n = kRootMinOrder;
-  e = launch_roots(ra, m, s);
+  e = launch_roots(ra, m, h->sms, s);
   if (e != cudaSuccess) return cuda_status(e);
   EigArgs a;
   memset(&a, 0, sizeof(a));

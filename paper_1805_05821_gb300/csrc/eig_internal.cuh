@@ -60,7 +60,7 @@ struct RootArgs {
   int *isc;
   int ld, min_n;
 };
-cudaError_t launch_roots(const RootArgs &a, int m, cudaStream_t s);
+cudaError_t launch_roots(const RootArgs &a, int m, int sms, cudaStream_t s);
 cudaError_t launch_invit(const EigArgs &e, bool after_qr, cudaStream_t s);
 cudaError_t launch_vectors(const EigArgs &e, int vgrid, cudaStream_t s);
 

@@ -18,7 +18,8 @@
 // the result does not depend on the order in which CTAs run.  They start on a circle around the mean
 // eigenvalue tr(H) / n whose radius is the geometric mean of |lambda - tr(H)/n|, from the determinant:
 // the Ritz values of a flow's snapshots lie near such a circle, and it takes 4 to 13 steps, 4.0 to 6.5
-// evaluations per eigenvalue (dense random matrices: 30 steps, 16 evaluations).
+// evaluations per eigenvalue (dense random matrices 7 steps at order 10, 15 at 48 and 30, FP32 ones included, at
+// 200).
 //
 // Why not the QR iteration: its chain of about 0.75 n^2 dependent 3 x 3 reflectors runs on one SM at
 // the latency of GB300's FP64 pipe (64 cycles an operation).  Here every eigenvalue is independent
@@ -285,6 +286,8 @@ __global__ void __launch_bounds__(512) roots_setup_kernel(RootArgs a) {
 
 // The start circle: its radius from the determinant of H - tr(H)/n.
 __global__ void __launch_bounds__(kRootThreads) roots_start_kernel(RootArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int n = a.isc[ISC_R], tid = threadIdx.x;
   if (a.isc[ISC_QR]) return;
   __shared__ HymanShared<float> hs;
@@ -304,8 +307,16 @@ __global__ void __launch_bounds__(kRootThreads) roots_start_kernel(RootArgs a) {
   }
 }
 
+// Steps after which a spectrum of n values is given up if none of them has converged: repeated eigenvalues,
+// whose corrections shrink by a third to two thirds a step.  (Where the iteration succeeds the first value
+// converges in step 4 to 9; the steps that are left out cost up to 12 us each at order 10, and the QR
+// iteration that follows them 260.)
+__device__ __forceinline__ int patience(int n) { return 8 + min(n, 32) / 8; }
+__device__ __forceinline__ bool given_up(const RootArgs &a, int n) { return a.left[patience(n) - 1] == n; }
+
 // The FP64 step after which no value was left, -1 if there is none
-__device__ __forceinline__ int last_step(const RootArgs &a) {
+__device__ __forceinline__ int last_step(const RootArgs &a, int n) {
+  if (given_up(a, n)) return -1;
   for (int k = 0; k < kRootSteps; ++k)
     if (a.left[k] == 0) return k;
   return -1;
@@ -332,6 +343,8 @@ __device__ __forceinline__ void correction(T pr, T pi, T qr, T qi, T sr, T si, T
 // takes 4 cycles where an FP64 one takes 64: 57 us a step at n = 255 against 131.  What FP32 makes of
 // a value only decides where the FP64 phase starts from: a value that it cannot improve stays.
 __global__ void __launch_bounds__(kRootThreads) roots_step32_kernel(RootArgs a, int it) {
+  pdl_wait();
+  pdl_trigger();
   const int n = a.isc[ISC_R], i = blockIdx.x;
   if (i >= n || a.isc[ISC_QR]) return;
   const int tid = threadIdx.x, K = a.ld;
@@ -380,8 +393,10 @@ __global__ void __launch_bounds__(kRootThreads) roots_step32_kernel(RootArgs a, 
 
 // Step `it` of the second phase, in FP64.
 __global__ void __launch_bounds__(kRootThreads) roots_step_kernel(RootArgs a, int it) {
+  pdl_wait();
+  pdl_trigger();
   const int n = a.isc[ISC_R], i = blockIdx.x;
-  if (i >= n || a.isc[ISC_QR] || (it > 0 && a.left[it - 1] == 0)) return;
+  if (i >= n || a.isc[ISC_QR] || (it > 0 && a.left[it - 1] == 0) || given_up(a, n)) return;
   const int tid = threadIdx.x, K = a.ld;
   const double *zri = a.zr + (it & 1) * K, *zii = a.zi + (it & 1) * K;
   double *zro = a.zr + ((it & 1) ^ 1) * K, *zio = a.zi + ((it & 1) ^ 1) * K;
@@ -430,9 +445,11 @@ __global__ void __launch_bounds__(kRootThreads) roots_step_kernel(RootArgs a, in
 
 // For each value the one nearest to its conjugate, and its nearest neighbour: a warp per value
 __global__ void __launch_bounds__(256) roots_pair_kernel(RootArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int n = a.isc[ISC_R], i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (a.isc[ISC_QR] || i >= n) return;
-  const int last = last_step(a);
+  const int last = last_step(a, n);
   if (last < 0) return;
   const double *zr = a.zr + ((last & 1) ^ 1) * a.ld, *zi = a.zi + ((last & 1) ^ 1) * a.ld;
   double best = 1e300, near = 1e300;
@@ -467,6 +484,7 @@ __global__ void __launch_bounds__(256) roots_pair_kernel(RootArgs a) {
 // isc[ISC_QR] asks for the QR iteration.  Whether each is as accurate as the QR iteration's decides the
 // inverse iteration (invit_kernel), which takes the pairs' means as they are stored here.
 __global__ void __launch_bounds__(512) roots_finish_kernel(RootArgs a) {
+  pdl_wait();
   const int n = a.isc[ISC_R], tid = threadIdx.x, K = a.ld;
   if (a.isc[ISC_QR]) return;
   __shared__ double zr[kMaxK], zi[kMaxK], red[32];
@@ -474,8 +492,8 @@ __global__ void __launch_bounds__(512) roots_finish_kernel(RootArgs a) {
   __shared__ int bad, last;
   if (tid == 0) {
     bad = 0;
-    last = last_step(a);
-    a.isc[ISC_ITS] = last < 0 ? kRootSteps : last + 1;
+    last = last_step(a, n);
+    a.isc[ISC_ITS] = last >= 0 ? last + 1 : given_up(a, n) ? patience(n) : kRootSteps;
   }
   __syncthreads();
   if (last < 0) {
@@ -524,17 +542,30 @@ __global__ void __launch_bounds__(512) roots_finish_kernel(RootArgs a) {
   if (tid == 0) a.isc[ISC_STATUS] = FOA_DMD_OK;
 }
 
-cudaError_t launch_roots(const RootArgs &a, int m, cudaStream_t s) {
+// Up to one CTA per SM the steps follow one another as programmatic dependent launches (each waits before it
+// reads anything), so that a step that finds nothing left to do costs little more than its launch:
+// order 10 332 -> 292 us, order 100 925 -> 838 us.  Beyond that the next step's waiting CTAs unbalance the
+// running one's second CTAs over the SMs (order 255 3.47 -> 3.64 ms).
+cudaError_t launch_roots(const RootArgs &a, int m, int sms, cudaStream_t s) {
   roots_setup_kernel<<<1, 512, 0, s>>>(a);
-  if (m >= a.min_n) {
-    roots_start_kernel<<<1, kRootThreads, 0, s>>>(a);
-    for (int it = 0; it < (m >= kRootMin32 ? kRootSteps32 : 0); ++it) roots_step32_kernel<<<m, kRootThreads, 0, s>>>(a, it);
-    static_assert(kRootSteps32 % 2 == 0, "the FP64 phase starts from buffer 0");
-    for (int it = 0; it < kRootSteps; ++it) roots_step_kernel<<<m, kRootThreads, 0, s>>>(a, it);
-    roots_pair_kernel<<<(m + 7) / 8, 256, 0, s>>>(a);
-    roots_finish_kernel<<<1, 512, 0, s>>>(a);
-  }
-  return cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
+  if (m < a.min_n) return e;
+  static_assert(kRootSteps32 % 2 == 0, "the FP64 phase starts from buffer 0");
+  auto go = [&](auto k, int grid, int block, auto... args) {
+    if (e != cudaSuccess) return;
+    if (m <= sms) {
+      e = launch_pdl(k, grid, block, 0, s, args...);
+    } else {
+      k<<<grid, block, 0, s>>>(args...);
+      e = cudaGetLastError();
+    }
+  };
+  go(roots_start_kernel, 1, kRootThreads, a);
+  for (int it = 0; it < (m >= kRootMin32 ? kRootSteps32 : 0); ++it) go(roots_step32_kernel, m, kRootThreads, a, it);
+  for (int it = 0; it < kRootSteps; ++it) go(roots_step_kernel, m, kRootThreads, a, it);
+  go(roots_pair_kernel, (m + 7) / 8, 256, a);
+  go(roots_finish_kernel, 1, 512, a);
+  return e;
 }
 
 }  // namespace foa

@@ -57,6 +57,17 @@ def test_which_iteration_found_the_eigenvalues(kind, m, tmp_path):
     g.close()
 
 
+@pytest.mark.parametrize("m", [10, 20, 50, 100])
+def test_repeated_eigenvalues_are_given_up_early(m, tmp_path):
+    """Five-fold eigenvalues: no value has converged after 8 + min(m, 32) / 8 steps, and no more are taken
+    before the QR iteration."""
+    from paper_1805_05821_gb300.foa_dmd import foa_dmd_test_eig_path
+    g = load_with(matrix("multiple", m, 7 * m), tmp_path / "h.ckpt")
+    assert g.eig(0.0)["status"] == 0
+    assert foa_dmd_test_eig_path(g.h) == (True, 8 + min(m, 32) // 8)
+    g.close()
+
+
 @pytest.mark.parametrize("m,e", [(128, -160), (40, -160), (128, 160), (128, -100), (128, 40), (128, -40)])
 def test_scale_decides_without_a_step(m, e, tmp_path):
     """Entries whose scale FP32 cannot hold go to the QR iteration before any step is tried; 2^+-40 does not."""
