@@ -374,7 +374,7 @@ int foa_dmd_host_free(void *ptr);
  * Many independent streams of uneven n and k_max advanced together (all FP32 or all BF16
  * storage).  batch_push advances every stream whose x pointer is non-NULL by one push
  * (Algorithm 4, p = 1 each) in a single persistent kernel launch; streams have their own
- * H-bar, beta, V and q.  x_dev: DEVICE array of S device pointers.  h_last_dev: device array
+ * H-bar, beta, V and q, and the same bits whichever other streams the batch holds or advances.  x_dev: DEVICE array of S device pointers.  h_last_dev: device array
  * of S doubles receiving h_{q,q-1} of each stream (NaN for inactive or failed streams).
  * Graph-capturable: all per-push decisions are read from device memory.
  * Per-stream statuses are read with foa_dmd_batch_get_state.

@@ -4,7 +4,7 @@
 //
 //   plan_kernel     reads every stream's device state and the caller's pointer array, decides
 //                   which streams push, and cuts each stream's passes into work items of whole
-//                   pipeline stages (128 KB to 8 MB of V, about six items a CTA);
+//                   pipeline stages (128 KB to 2 MB of V, by the stream's own size);
 //   prep_kernel     beta_pre of every active stream (Alg. 1), one CTA per stream;
 //   bpass_kernel    pass A, then pass B, then pass C (pre-vector, CGS2, norm; Alg. 1) of all streams, one
 //                   launch per pass: two CTAs of 256 threads per SM take items from a counter;
@@ -40,12 +40,15 @@ constexpr int kStageCols = 256;             // R * j <= this while R > 1: stages
 constexpr int kRingBytes = 102400;          // the stage ring of a CTA (two 50 KB slots hold j <= 399)
 constexpr int kMaxBSlots = 6;
 constexpr int kCf = 640;                    // padded coefficient vector (>= 16 * 32 + 32)
-// V bytes per work item.  The CTAs take items from a counter, so a pass ends unevenly by up to one item
-// a CTA, while every item fills the ring anew and writes its partial sums (about 4 us): six items a CTA,
-// within these limits.  With 8 MB throughout, a round of 48 streams (16k to 1M values, 1.9 GB of V)
-// was 240 items for 304 CTAs: 438 us a pass, now 363 us.
-constexpr int64_t kItemBytesMax = 8ll << 20, kItemBytesMin = 128ll << 10;
-constexpr int kItemsPerCta = 6;
+// V bytes per work item: a share of the stream's own V, within limits, and nothing of the other streams': an item's
+// ends decide where FP32 column sums are folded and how the FP64 ones are grouped, so a stream has the same
+// bits in any company.  The CTAs take items from a counter: a pass ends unevenly by up to one item a CTA,
+// while every item fills the ring anew and writes its partial sums (about 4 us).  ms from creation to
+// states for 48 streams of 16k to 1M values (120 rounds, 1.9 GB of V) / 3 of 60k to 960k / 20 of 20k to 200k:
+//   share 1/96 149.1 / 19.0 / 20.6, 1/64 146.6 / 23.2 / 21.2, 1/128 152.9 / 17.1 / 21.0, 1/32 up to 8 MB
+//   160.4 / 36.7 / 25.4; 8 MB throughout 178.0 / 109.3 / 94.2; by the round's total bytes 145.5 / 19.7 / 23.0.
+constexpr int64_t kItemBytesMax = 2ll << 20, kItemBytesMin = 128ll << 10;
+constexpr int kItemShare = 96;
 constexpr int kItemStages = 256;            // at most this many stages ...
 constexpr int kStreamItems = 512;           // ... and this many items of one stream (summed by one CTA)
 enum { PH_A = 0, PH_B = 1, PH_C = 2, PH_APP = 3, NPH = 4 };
@@ -94,7 +97,6 @@ struct BatchArgs {
   double *vec;         // pools of pre/h/s
   double *part;        // partials of a pass's items, by item
   int32_t pstride;     // doubles of one item's partials
-  int32_t ctas;        // CTAs of a pass
   const void *const *x;  // caller's pointers (device array of S)
   double *h_last;      // caller's output array (device, S)
   double tol;
@@ -110,27 +112,21 @@ __host__ __device__ __forceinline__ int stage_tiles(int j) {
   return R;
 }
 
-// stages of one item for `goal` bytes
-__host__ __device__ __forceinline__ int item_stages(int64_t goal, int64_t stage_bytes) {
-  const int64_t cs = goal / stage_bytes;
-  return cs > kItemStages ? kItemStages : cs < 1 ? 1 : int(cs);
+// stages of one work item of a stream with ntiles tiles at basis size j
+__host__ __device__ __forceinline__ int item_stages(int ntiles, int j, int ssize) {
+  const int R = stage_tiles(j), nstages = (ntiles + R - 1) / R;
+  const int64_t stage_bytes = int64_t(R) * kTile * (j > 0 ? j : 1) * ssize;
+  int64_t goal = nstages * stage_bytes / kItemShare;
+  goal = goal < kItemBytesMin ? kItemBytesMin : goal > kItemBytesMax ? kItemBytesMax : goal;
+  int64_t cs = goal / stage_bytes;
+  if (cs > kItemStages) cs = kItemStages;
+  const int64_t least = (nstages + kStreamItems - 1) / kStreamItems;
+  return int(cs < least ? least : cs < 1 ? 1 : cs);
 }
 
 __global__ void plan_kernel(BatchArgs a, int ssize) {
   const int S = a.S;
   extern __shared__ int32_t cnt[];  // NPH * S counts
-  __shared__ unsigned long long bytes;
-  if (threadIdx.x == 0) bytes = 0ull;
-  __syncthreads();
-  for (int s = threadIdx.x; s < S; s += blockDim.x) {  // V bytes of this round
-    const BState &b = a.st[s];
-    const StreamDesc d = a.sd[s];
-    if (a.x[s] && !b.stopped && b.q < d.kmax)
-      atomicAdd(&bytes, (unsigned long long)(int64_t(d.ntiles) * kTile * max(b.q, 1) * ssize));
-  }
-  __syncthreads();
-  int64_t goal = int64_t(bytes) / (int64_t(a.ctas) * kItemsPerCta);
-  goal = goal < kItemBytesMin ? kItemBytesMin : goal > kItemBytesMax ? kItemBytesMax : goal;
   for (int s = threadIdx.x; s < S; s += blockDim.x) {
     const StreamDesc d = a.sd[s];
     BState &b = a.st[s];
@@ -147,9 +143,7 @@ __global__ void plan_kernel(BatchArgs a, int ssize) {
     Plan p;
     p.R = stage_tiles(j);
     p.nstages = (d.ntiles + p.R - 1) / p.R;
-    const int64_t stage_bytes = int64_t(p.R) * kTile * (j > 0 ? j : 1) * ssize;
-    p.cs = item_stages(goal, stage_bytes);
-    p.cs = max(p.cs, (p.nstages + kStreamItems - 1) / kStreamItems);
+    p.cs = item_stages(d.ntiles, j, ssize);
     p.nchunks = (p.nstages + p.cs - 1) / p.cs;
     a.plan[s] = p;
     const bool first = (j == 0);
@@ -636,16 +630,13 @@ static void batch_free(foa_dmd_batch *b) {
     if (p) cudaFree(p);
 }
 
-// the largest number of work items of kItemBytesMax a pass of this stream can have (over every basis size j)
+// the largest number of work items a pass of this stream can have (over every basis size j)
 static int32_t max_items(int32_t ntiles, int32_t kmax, int es) {
   int32_t best = 1;
   for (int j = 0; j < kmax; ++j) {
-    const int R = stage_tiles(j);
-    const int64_t nstages = (ntiles + R - 1) / R;
-    const int64_t stage_bytes = int64_t(R) * kTile * (j > 0 ? j : 1) * es;
-    const int64_t cs = item_stages(kItemBytesMax, stage_bytes);
-    const int64_t nc = (nstages + cs - 1) / cs;
-    if (nc > best) best = int32_t(nc);
+    const int R = stage_tiles(j), nstages = (ntiles + R - 1) / R, cs = item_stages(ntiles, j, es);
+    const int32_t nc = (nstages + cs - 1) / cs;
+    if (nc > best) best = nc;
   }
   return best;
 }
@@ -693,10 +684,6 @@ extern "C" int foa_dmd_batch_create(int32_t S, const int64_t *n, const int32_t *
     items += max_items(d.ntiles, d.kmax, es);
     if (d.kmax + 1 > pstride) pstride = d.kmax + 1;
   }
-  // Items of a pass: a stream's are as many as max_items where they have kItemStages stages or
-  // kItemBytesMax bytes, else at most 1.5 x its share of kItemsPerCta a CTA, plus one (a stage is at most
-  // half of kItemBytesMin, so whole stages fill two thirds of the goal).
-  items += 3 * int64_t(sms) * kItemsPerCta + S;
   b->pstride = pstride;
   cudaError_t e = cudaSuccess;
 #define BAL(p, bytes)                                         \
@@ -757,7 +744,6 @@ extern "C" int foa_dmd_batch_push(foa_dmd_batch_t *b, const void *const *x_dev, 
   a.vec = b->vec;
   a.part = b->part;
   a.pstride = b->pstride;
-  a.ctas = 2 * b->sms;
   a.x = x_dev;
   a.h_last = h_last_dev;
   a.tol = b->tol;
