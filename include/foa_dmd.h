@@ -337,12 +337,13 @@ int foa_dmd_push_block(foa_dmd_t *h, const void *X_dev, int32_t p, int64_t ld, i
  * Autotuner of the streaming-pass launch geometry (no counterpart in the paper).  For every pass
  * kind the handle's options use (A/B/C, or the two passes of reorth = 2) and every j bucket up to
  * k_max (upper ends 8, 16, 32, 64, 128, 192, 256, 320, 384, 448, 512), times each candidate
- * (V bytes per pipeline stage 16/32/64 KB x V bytes in flight per CTA 64/96/144/192 KB x one or two
+ * (V bytes per pipeline stage 16/32/64 KB, FP64 48 KB too, x V bytes in flight per CTA 64/96/144/192 KB x one or two
  * CTAs per SM x, for the FP32/BF16 passes with column dots, the register-held or the shared-
  * memory form of the stage) on the handle's own buffers, over a prefix of V of about 2 GB, median
  * of three launches, and keeps the fastest; later pushes of the handle launch with it.
  *   cache_path: NULL, or a text file.  Choices found there for (device arch, dtype, floor(log2 n),
- *               kind, bucket) are used without timing; new choices are appended.
+ *               kind, bucket) are used without timing, those of another version of the kernels are passed
+ *               over; new choices are appended.
  *   flags:      bit 0 = time again even where the cache has a choice.
  * The handle must hold no snapshots (q == 0, e.g. right after create or reset): tuning overwrites
  * V, H-bar, beta and the working vector, and clears them again before returning.  Errors:

@@ -35,7 +35,7 @@ Geometry default_geometry(int dtype) {
 // Shared-memory layout and grid of one streaming pass (the launch geometry depends only on the
 // dtype, the pass kind, jcap and n, so identical pushes always get identical launches).
 bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n, int ntiles, int sms, PassArgs &a,
-                    int &grid) {
+                    int &grid, int *ctas_per_sm) {
   const int s = dtype_size(dtype), cs = compute_size(dtype);
   const bool lag = (mode == PASS_A2 || mode == PASS_FIN);
   const bool basex = (mode == PASS_A || mode == PASS_FIRST);
@@ -108,6 +108,7 @@ bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n,
   a.jcap = jcap;
   a.nstages = (ntiles + R - 1) / R;
   const int per_sm = two ? 2 : 1;
+  if (ctas_per_sm) *ctas_per_sm = per_sm;
   grid = a.nstages < sms * per_sm ? a.nstages : sms * per_sm;
   return true;
 }

@@ -119,7 +119,7 @@ double default_tol(int dtype);
 int max_kmax_for(int dtype);
 Geometry default_geometry(int dtype);
 bool make_pass_geom(const Geometry &g, int dtype, int mode, int jcap, int64_t n, int ntiles, int sms, PassArgs &a,
-                    int &grid);
+                    int &grid, int *ctas_per_sm = nullptr);
 int launch_pass_h(foa_dmd *h, int mode, int jcap, const void *x, const double *coef, bool batch,
                   foa_dmd_push_info *info_out);
 int enqueue_push(foa_dmd *h, const void *x, bool batch, foa_dmd_push_info *info_out);

@@ -10,7 +10,6 @@
 // bucket) that later handles read instead of timing again.
 #include <cmath>
 #include <cstdio>
-#include <cstdlib>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -89,17 +88,23 @@ int log2_floor(int64_t n) {
   return l;
 }
 
-// Cache lines: "foa_dmd_tune arch dtype log2n kind bucket stage inflight ctas variant ms"
+// Cache lines: "foa_dmd_tune vVERSION arch dtype log2n kind bucket stage inflight ctas variant ms".  Lines of
+// another version, or of before there were any, are passed over: the kernels they were timed on launch
+// differently now (FP64 passes with two CTAs per SM, buckets timed inside their range).
+constexpr int kTuneVersion = 2;
+
 void load_cache(foa_dmd *h, const char *path, int arch, int nb) {
   FILE *f = fopen(path, "r");
   if (!f) return;
-  char tag[32];
-  int a, dt, l2, kind, b, ctas, variant;
+  char line[256];
+  int v, a, dt, l2, kind, b, ctas, variant;
   long long stage, inflight;
   double ms;
-  while (fscanf(f, "%31s %d %d %d %d %d %lld %lld %d %d %lf", tag, &a, &dt, &l2, &kind, &b, &stage, &inflight, &ctas,
-                &variant, &ms) == 11) {
-    if (strcmp(tag, "foa_dmd_tune") != 0 || a != arch || dt != h->dtype || l2 != nb) continue;
+  while (fgets(line, sizeof(line), f)) {
+    if (sscanf(line, "foa_dmd_tune v%d %d %d %d %d %d %lld %lld %d %d %lf", &v, &a, &dt, &l2, &kind, &b, &stage, &inflight,
+               &ctas, &variant, &ms) != 11)
+      continue;
+    if (v != kTuneVersion || a != arch || dt != h->dtype || l2 != nb) continue;
     if (kind < 0 || kind >= kTuneKinds || b < 0 || b >= kTuneBuckets) continue;
     if (stage < 4096 || stage > (1 << 20) || inflight < 4096 || inflight > (1 << 20) || ctas < 1 || ctas > 2) continue;
     Geometry g = h->geom;
@@ -154,7 +159,12 @@ extern "C" int foa_dmd_autotune(foa_dmd_t *h, const char *cache_path, int32_t fl
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   std::vector<Candidate> cands;
+  // the default stage first: where another one is the same launch at the timed j (and not all over the
+  // bucket), the default stands for both
+  std::vector<int64_t> stages = {h->geom.stage_bytes};
   for (int64_t st : {16384, 32768, 65536})
+    if (st != h->geom.stage_bytes) stages.push_back(st);
+  for (int64_t st : stages)
     for (int64_t inf : {65536, 98304, 147456, 196608})
       for (int c : {1, 2})
         for (int v : {0, 1}) cands.push_back({st, inf, c, v});
@@ -165,8 +175,12 @@ extern "C" int foa_dmd_autotune(foa_dmd_t *h, const char *cache_path, int32_t fl
     const int mode = kKindMode[k];
     for (int b = 0; b < nbuckets && rc == FOA_DMD_OK; ++b) {
       if (h->tuned_ok[k][b] && !(flags & 1)) continue;
-      int j = kTuneEdges[b] < jmax ? kTuneEdges[b] : jmax;
-      if (j < 1) j = 1;
+      // timed in the middle of the bucket: at its upper end, a power of two or three times one, stages of 32 and
+      // 48 KB hold the same tiles
+      const int below = b ? kTuneEdges[b - 1] : 0;
+      int jtop = kTuneEdges[b] < jmax ? kTuneEdges[b] : jmax;
+      if (jtop < 1) jtop = 1;
+      const int j = below + (jtop - below + 1) / 2;
       // time on a prefix of V large enough to stream well past L2 (about 2 GB), at most all of it
       const int64_t tile_bytes = int64_t(kTile) * j * s;
       int64_t tiles = int64_t(2) << 30;
@@ -189,6 +203,7 @@ extern "C" int foa_dmd_autotune(foa_dmd_t *h, const char *cache_path, int32_t fl
         PassArgs a;
         memset(&a, 0, sizeof(a));
         int grid = 0;
+        if (!make_pass_geom(g, h->dtype, mode, jtop, n_t, int(tiles), sms, a, grid)) continue;  // must fit all of it
         if (!make_pass_geom(g, h->dtype, mode, j, n_t, int(tiles), sms, a, grid)) continue;
         char key[96];
         snprintf(key, sizeof(key), "%d/%d/%d/%d/%d", a.R, a.slots, grid, a.smem_total, c.variant);
@@ -251,7 +266,7 @@ extern "C" int foa_dmd_autotune(foa_dmd_t *h, const char *cache_path, int32_t fl
       h->tuned[k][b] = bestg;
       h->tuned_ok[k][b] = true;
       if (cache)
-        fprintf(cache, "foa_dmd_tune %d %d %d %d %d %lld %lld %d %d %.6f\n", arch, h->dtype, nb, k, b,
+        fprintf(cache, "foa_dmd_tune v%d %d %d %d %d %d %lld %lld %d %d %.6f\n", kTuneVersion, arch, h->dtype, nb, k, b,
                 (long long)bestg.stage_bytes, (long long)bestg.inflight_bytes, bestg.max_ctas_per_sm, bestg.variant,
                 best);
     }
@@ -282,7 +297,12 @@ extern "C" int foa_dmd_tuned_geometry(foa_dmd_t *h, int32_t kind, int32_t j, int
   const Geometry &g = geom_for(h, kKindMode[kind], j);
   if (stage_bytes) *stage_bytes = g.stage_bytes;
   if (inflight_bytes) *inflight_bytes = g.inflight_bytes;
-  if (ctas_per_sm) *ctas_per_sm = g.max_ctas_per_sm;
+  if (ctas_per_sm) {
+    PassArgs a;
+    int grid = 0;
+    *ctas_per_sm = g.max_ctas_per_sm;  // the limit; what this pass launches with, where it fits at all
+    make_pass_geom(g, h->dtype, kKindMode[kind], j, h->n, h->ntiles, h->sms, a, grid, ctas_per_sm);
+  }
   if (variant) *variant = g.variant;
   if (tuned) *tuned = h->tuned_ok[kind][tune_bucket(j)] ? 1 : 0;
   return FOA_DMD_OK;
