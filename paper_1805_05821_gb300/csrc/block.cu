@@ -4,7 +4,7 @@
 //   BLK_B  (one pass over V)  W = X_b - V C1,  C2 = V^T W,  C = C1 + C2
 //   BLK_C  (one pass over V)  W = W - V C2,    G = W^T W, then G = R1^T R1 (Cholesky, FP64)
 //   blockq1 (rows of W only)  W1 = W R1^-1 (FP64), G2 = W1^T W1 = R2^T R2, R = R2 R1, breakdown test,
-//                             beta block column [C; R]; without the rows where R1 is well conditioned
+//                             beta block column [C; R]
 //   blockh                    Hbar columns by forward substitution, one warp per row
 //   blockq2 (rows of W only)  Q = W R^-1 -> V columns j .. j+P-1
 // V is read three times per block instead of three times per snapshot.  The three passes over V
@@ -24,9 +24,8 @@ namespace blk {
 
 // The second Cholesky step and the scalar part of the block.  W1 = W R1^-1 on the leading m1 columns
 // (FP64, by reciprocals), G2 = W1^T W1, and in the last CTA: R2, R = R2 R1, the breakdown test, the
-// beta block column, the device state.  The rows cost 20 FP64 operations each at 2 a clock and SM; where
-// R1 is well conditioned (kWellKappa) R2 = I is as good and one CTA does the scalar part alone.  (With
-// divisions, the rows always, and the Hbar columns in the last CTA: 502 us a block at n = 4194304.)
+// beta block column, the device state.  The rows cost 20 FP64 operations each at 2 a clock and SM, which bounds
+// the kernel.  (With divisions, W1 stored and the Hbar columns in the last CTA: 502 us a block at n = 4194304.)
 template <int P>
 __global__ void __launch_bounds__(256) blockq1_kernel(BlockArgs a, foa_dmd_push_info *info_out) {
   constexpr int NG = P * (P + 1) / 2;
@@ -37,63 +36,54 @@ __global__ void __launch_bounds__(256) blockq1_kernel(BlockArgs a, foa_dmd_push_
   if (!a.st->active) return;
   BlockState *bs = a.bs;
   const int m1 = __ldcg(&bs->m1);
-  const bool well = __ldcg(&bs->well) != 0;
-  if (well) {
-    if (blockIdx.x != 0) return;
-  } else {
-    double R1[P * P], iv[P];
+  double R1[P * P], iv[P];
 #pragma unroll
-    for (int i = 0; i < P * P; ++i) R1[i] = __ldcg(&bs->R1[(i % P) + (i / P) * kMaxP]);
+  for (int i = 0; i < P * P; ++i) R1[i] = __ldcg(&bs->R1[(i % P) + (i / P) * kMaxP]);
 #pragma unroll
-    for (int c = 0; c < P; ++c) iv[c] = c < m1 ? 1.0 / R1[c + c * P] : 0.0;
-    double g[NG];
+  for (int c = 0; c < P; ++c) iv[c] = c < m1 ? 1.0 / R1[c + c * P] : 0.0;
+  double g[NG];
 #pragma unroll
-    for (int i = 0; i < NG; ++i) g[i] = 0.0;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t r = int64_t(blockIdx.x) * blockDim.x + tid; r < a.nrows; r += stride) {
-      double w1[P];
+  for (int i = 0; i < NG; ++i) g[i] = 0.0;
+  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+  for (int64_t r = int64_t(blockIdx.x) * blockDim.x + tid; r < a.nrows; r += stride) {
+    double w1[P];
 #pragma unroll
-      for (int c = 0; c < P; ++c) {
-        double t = a.W[int64_t(c) * a.nrows + r];
+    for (int c = 0; c < P; ++c) {
+      double t = a.W[int64_t(c) * a.nrows + r];
 #pragma unroll
-        for (int k = 0; k < c; ++k) t -= w1[k] * R1[k + c * P];
-        w1[c] = t * iv[c];
-      }
-      int q = 0;
-#pragma unroll
-      for (int k = 0; k < P; ++k)
-#pragma unroll
-        for (int l = k; l < P; ++l, ++q) g[q] += w1[k] * w1[l];
+      for (int k = 0; k < c; ++k) t -= w1[k] * R1[k + c * P];
+      w1[c] = t * iv[c];
     }
+    int q = 0;
 #pragma unroll
-    for (int i = 0; i < NG; ++i) {
-      const double t = warp_sum(g[i]);
-      if (lane == 0) red[warp * NG + i] = t;
-    }
-    __syncthreads();
-    if (tid < NG) {
-      double t = 0.0;
-      for (int w = 0; w < 8; ++w) t += red[w * NG + tid];
-      dot[tid] = t;
-    }
-    __syncthreads();
-    if (!grid_reduce<256>(a.partials, a.gpart, a.gcount, &bs->ticket[3], NG, dot, NG, sflag + 2, tid)) return;
+    for (int k = 0; k < P; ++k)
+#pragma unroll
+      for (int l = k; l < P; ++l, ++q) g[q] += w1[k] * w1[l];
   }
+#pragma unroll
+  for (int i = 0; i < NG; ++i) {
+    const double t = warp_sum(g[i]);
+    if (lane == 0) red[warp * NG + i] = t;
+  }
+  __syncthreads();
+  if (tid < NG) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w * NG + tid];
+    dot[tid] = t;
+  }
+  __syncthreads();
+  if (!grid_reduce<256>(a.partials, a.gpart, a.gcount, &bs->ticket[3], NG, dot, NG, sflag + 2, tid)) return;
   // ---------------- the last CTA
   const int j = a.j;
   const int K = a.kmax;
   if (tid == 0) {
     double G2[kMaxP * kMaxP];
     for (int i = 0; i < kMaxP * kMaxP; ++i) G2[i] = 0.0;
-    int m = m1, q = 0;
-    if (well) {
-      for (int i = 0; i < kMaxP * kMaxP; ++i) bs->R2[i] = (i % (kMaxP + 1) == 0) ? 1.0 : 0.0;
-    } else {
-      for (int k = 0; k < P; ++k)
-        for (int l = k; l < P; ++l, ++q)
-          if (l < m1) G2[k + l * kMaxP] = G2[l + k * kMaxP] = dot[q];
-      m = m1 > 0 ? chol_up(m1, G2, bs->R2) : 0;
-    }
+    int q = 0;
+    for (int k = 0; k < P; ++k)
+      for (int l = k; l < P; ++l, ++q)
+        if (l < m1) G2[k + l * kMaxP] = G2[l + k * kMaxP] = dot[q];
+    const int m = m1 > 0 ? chol_up(m1, G2, bs->R2) : 0;
     // R = R2 R1: rows r < m for every column c (columns past the factored block keep their
     // coefficients on the factored directions)
     for (int i = 0; i < kMaxP * kMaxP; ++i) bs->R[i] = 0.0;
@@ -137,7 +127,6 @@ __global__ void __launch_bounds__(256) blockq1_kernel(BlockArgs a, foa_dmd_push_
   // results of the columns (the Hbar columns themselves: blockh_kernel)
   const int ncols = nc + ((status == FOA_DMD_EBREAKDOWN) ? 1 : 0);
   if (tid == 0) {
-    tri_inv(nc, bs->R, bs->Rinv);
     for (int i = 0; i < ncols; ++i) {
       const double bjj = i == 0 ? a.B[int64_t(j - 1) * (K + 1)] : bs->R[(i - 1) * (kMaxP + 1)];
       foa_dmd_push_info inf;
@@ -211,18 +200,17 @@ __global__ void __launch_bounds__(256) blockh_kernel(BlockArgs a) {
   }
 }
 
-// Q = W R^-1 -> V columns j .. j+ncommit-1 (row-tiled), rows beyond n zero.  A thread takes four rows
-// (16-byte accesses).  Where R1 is well conditioned the products with R^-1 are formed in FP32 pairs
-// (each entry of R^-1 as the sum of two floats, exact products and sums by fma and two-sum): 2^-45
-// of sum |w_k r_kc| <= 512 |q_c| per entry, far below the rounding to storage that follows, at FP32's
-// rate; otherwise by two FP64 substitutions.  (FP64 with divisions: 323 us a block at n = 4194304; block push of 256 snapshots there 149 -> 100 ms with the changes here.)
+// Q = W R^-1 -> V columns j .. j+ncommit-1 (row-tiled), rows beyond n zero: two FP64 substitutions a row, by
+// reciprocals, rounded to storage once; FP64's 2 operations a clock and SM bound them.  A thread takes four rows
+// (16-byte accesses).  (From a stored FP64 W1, with divisions, one row a thread: 323 us a block at n = 4194304.
+// A block of 4 there 2330 us with that, 1960 now; with R^-1 in FP32 pairs and one Cholesky step where R1 is well
+// conditioned 1560, but fewer bits, and none at all where R^-1 leaves FP32's range.)
 template <typename S, int P>
 __global__ void __launch_bounds__(256) blockq2_kernel(BlockArgs a) {
   if (!a.st->active) return;
   const BlockState *bs = a.bs;
   const int nc = __ldcg(&bs->ncommit);
   if (nc == 0) return;
-  const bool well = __ldcg(&bs->well) != 0;
   S *V = static_cast<S *>(const_cast<void *>(a.V));
   const int64_t stride = 4 * int64_t(gridDim.x) * blockDim.x;
   const int64_t first = 4 * (int64_t(blockIdx.x) * blockDim.x + threadIdx.x);
@@ -240,41 +228,6 @@ __global__ void __launch_bounds__(256) blockq2_kernel(BlockArgs a) {
     }
     st4(V + ((r >> 5) * a.kmax + a.j + c) * kTile + (r & 31), v);
   };
-  if (well) {
-    float rh[P][P], rl[P][P];
-#pragma unroll
-    for (int c = 0; c < P; ++c)
-#pragma unroll
-      for (int k = 0; k <= c; ++k) {
-        const double v = __ldcg(&bs->Rinv[k + c * kMaxP]);
-        rh[k][c] = float(v);
-        rl[k][c] = float(v - double(rh[k][c]));
-      }
-    for (int64_t r = first; r < a.nrows; r += stride) {
-      float w[P][4];
-      load(r, w);
-#pragma unroll
-      for (int c = 0; c < P; ++c) {
-        float q[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          float s = __fmul_rn(w[0][u], rh[0][c]);
-          float e = fmaf(w[0][u], rl[0][c], fmaf(w[0][u], rh[0][c], -s));
-#pragma unroll
-          for (int k = 1; k <= c; ++k) {
-            const float p = __fmul_rn(w[k][u], rh[k][c]);
-            const float pe = fmaf(w[k][u], rl[k][c], fmaf(w[k][u], rh[k][c], -p));
-            const float t = __fadd_rn(s, p), bb = __fsub_rn(t, s);
-            e = __fadd_rn(e, __fadd_rn(pe, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(p, bb))));
-            s = t;
-          }
-          q[u] = __fadd_rn(s, e);
-        }
-        if (c < nc) store(r, c, q);
-      }
-    }
-    return;
-  }
   double R1[P * P], R2[P * P], i1[P], i2[P];
 #pragma unroll
   for (int i = 0; i < P * P; ++i) {

@@ -19,11 +19,6 @@ __host__ __device__ inline double unit_roundoff(int dtype) {
   return dtype == FOA_DMD_F64 ? 0x1p-53 : dtype == FOA_DMD_F32 ? 0x1p-24 : 0x1p-8;
 }
 
-// One Cholesky QR step leaves Q's orthogonality at about u_fp64 kappa(R1)^2.  Below this Frobenius
-// condition number of R1 that is 2^-35, a thousandth of the FP32 rounding that Q gets when it is
-// stored, and the second step (which brings it to u_fp64) changes nothing that is kept: it is left out.
-constexpr double kWellKappa = 512.0;
-
 struct BlockState {
   int32_t j;        // basis size before the block
   int32_t pb;       // snapshots in the block
@@ -35,8 +30,6 @@ struct BlockState {
   double xnorm[kMaxP];
   double R1[kMaxP * kMaxP], R2[kMaxP * kMaxP], R[kMaxP * kMaxP];
   double G[kMaxP * kMaxP];
-  double Rinv[kMaxP * kMaxP];  // R^-1, with R = R2 R1
-  int32_t well;                // R1 is so well conditioned that one Cholesky step does (kWellKappa)
 };
 
 struct BlockArgs {
@@ -74,24 +67,6 @@ __device__ inline int chol_up(int p, const double *G, double *R) {
     }
   }
   return p;
-}
-
-// inverse of the leading p x p block of the upper triangular R
-__device__ inline void tri_inv(int p, const double *R, double *I) {
-  for (int i = 0; i < kMaxP * kMaxP; ++i) I[i] = 0.0;
-  for (int c = 0; c < p; ++c) {
-    I[c + c * kMaxP] = 1.0 / R[c + c * kMaxP];
-    for (int r = c - 1; r >= 0; --r) {
-      double t = 0.0;
-      for (int k = r + 1; k <= c; ++k) t -= R[r + k * kMaxP] * I[k + c * kMaxP];
-      I[r + c * kMaxP] = t * I[r + r * kMaxP];
-    }
-  }
-}
-__device__ inline double frobenius(const double *M) {
-  double t = 0.0;
-  for (int i = 0; i < kMaxP * kMaxP; ++i) t += M[i] * M[i];
-  return sqrt(t);
 }
 
 // Shape of a block pass at basis size j: T threads a CTA (256: two CTAs per SM, basis up to 256

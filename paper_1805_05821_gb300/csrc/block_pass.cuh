@@ -381,12 +381,6 @@ __global__ void __launch_bounds__(T, 512 / T) block_pass_kernel(const BlockArgs 
       for (int k = 0; k < P; ++k)
         for (int l = 0; l < P; ++l) bs->G[k + l * kMaxP] = dot[k + l * P];
       bs->m1 = chol_up(P, bs->G, bs->R1);
-      int well = 0;
-      if (bs->m1 == P) {
-        tri_inv(P, bs->R1, bs->Rinv);
-        well = frobenius(bs->R1) * frobenius(bs->Rinv) <= kWellKappa;
-      }
-      bs->well = well;
     }
     named_bar_sync(1, T);
     // C = C1 + C2 (C2 was the row sweep's coefficient)

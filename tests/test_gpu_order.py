@@ -20,6 +20,10 @@ CASES = {"f32": ("f32", 400001, 140, 1, 0), "bf16": ("bf16", 400001, 150, 1, 0),
          "f32_two_pass": ("f32", 400001, 140, 2, 0), "bf16_two_pass": ("bf16", 100003, 70, 2, 0)}
 
 
+# dtype, n, N, block: the Cholesky QR of a block works in FP64 up to the rounding of Q to storage
+BLOCKS = {"f32_block4": ("f32", 100000, 69, 4), "f32_block2": ("f32", 40000, 41, 2), "bf16_block4": ("bf16", 40000, 41, 4)}
+
+
 def snapshot_rows(n, N):
     """x_0 noise, x_t = 7/8 x_{t-1} + noise, in FP32: integer arithmetic and separately rounded operations."""
     i = np.arange(n, dtype=np.uint64)
@@ -39,6 +43,20 @@ def record(F, dt, n, N, reorth, form):
     for x in snapshot_rows(n, N):
         st, info = g.push(torch.from_numpy(x).cuda().to(td))
         assert st == 0, info
+    return result(g, dt, N)
+
+
+def record_block(F, dt, n, N, block):
+    import torch
+    g = F.FoaDMD(n, N, dt)
+    X = torch.from_numpy(np.stack(list(snapshot_rows(n, N)))).cuda().to({"f32": torch.float32, "bf16": torch.bfloat16}[dt])
+    st, infos = g.push_block(X, block)
+    assert st == 0, infos
+    return result(g, dt, N)
+
+
+def result(g, dt, N):
+    import torch
     q, _, H, B = g.state()
     assert q == N
     V = g.basis(0, N).contiguous()
@@ -48,7 +66,7 @@ def record(F, dt, n, N, reorth, form):
     return {"bits": bits, "sub": sub, "last": [float(v) for v in B[:N, N - 1]]}
 
 
-@pytest.mark.parametrize("name", sorted(CASES))
+@pytest.mark.parametrize("name", sorted(CASES) + sorted(BLOCKS))
 def test_order_of_the_sums(name):
     import torch
     from paper_1805_05821_gb300 import build, foa_dmd
@@ -56,9 +74,27 @@ def test_order_of_the_sums(name):
     if torch.cuda.get_device_properties(0).multi_processor_count != 152:
         pytest.skip("the stages are dealt over 152 SMs")
     want = json.load(open(GOLDEN))[name]
-    got = record(foa_dmd, *CASES[name])
+    got = record(foa_dmd, *CASES[name]) if name in CASES else record_block(foa_dmd, *BLOCKS[name])
     bad = [c for c in range(len(want["bits"])) if want["bits"][c] != got["bits"][c]]
     for key in ("sub", "last"):
         w, g = np.array(want[key]), np.array(got[key])
         assert np.abs(g - w).max() <= 1e-12 * np.abs(w).max(), (key, np.abs(g - w).max())
     assert not bad, f"columns {bad[:8]} of {len(want['bits'])} differ in their bits"
+
+
+@pytest.mark.parametrize("block", [2, 4])
+def test_block_of_tiny_values(block):
+    """A block whose R^-1 lies beyond FP32 (entries of about 1e-40): its columns are as orthonormal as entries
+    with steps of 2^-149 allow, 2^-149 / 1e-40 = 1.4e-5 each, twice over 64 rows and the three passes."""
+    import torch
+    from paper_1805_05821_gb300 import build, foa_dmd
+    build.build()
+    n = 64
+    r = np.random.default_rng(block)
+    X = np.concatenate([r.standard_normal((1, n)), 1e-40 * r.standard_normal((block, n))]).astype(np.float32)
+    g = foa_dmd.FoaDMD(n, 1 + block, "f32")
+    st, infos = g.push_block(torch.from_numpy(X).cuda(), block)
+    assert st == 0 and g.state()[0] == 1 + block, infos
+    V = g.basis(0, 1 + block).double().cpu().numpy()
+    assert np.abs(V @ V.T - np.eye(1 + block)).max() <= 6 * 64 * 2.0 ** -149 / 1e-40
+    g.close()
