@@ -456,83 +456,28 @@ __global__ void __launch_bounds__(kThreads, pass_min_blocks<S, NC>()) pass_kerne
           const int c1 = min(j, c0 + cpg);
           for (int row = (G == 1 ? tid : tid % RS); row < RS; row += (G == 1 ? kConsumers : RS)) {
             const S *vr = vs + (row >> 5) * (kTile * j) + (row & 31);
-            double accd = 0.0;
-            float accf = 0.f;
-            if constexpr (kFp64) {
-              double b0 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0;
-              int c = c0;
-              for (; c + 4 <= c1; c += 4) {
-                b0 = fma(to_c(vr[(c + 0) * kTile]), cf[c + 0], b0);
-                b1 = fma(to_c(vr[(c + 1) * kTile]), cf[c + 1], b1);
-                b2 = fma(to_c(vr[(c + 2) * kTile]), cf[c + 2], b2);
-                b3 = fma(to_c(vr[(c + 3) * kTile]), cf[c + 3], b3);
-              }
-              for (; c < c1; ++c) b0 = fma(to_c(vr[c * kTile]), cf[c], b0);
-              accd = (b0 + b1) + (b2 + b3);
-            } else {
-              // FP32: four independent chains over the thread's columns (no FP64 in the row loop:
-              // the FP64 pipe of this part is ~1/64 of FP32)
-              float b[8];
-    #pragma unroll
-              for (int u = 0; u < 8; ++u) b[u] = 0.f;
-              int c = c0;
-              for (; c + 8 <= c1; c += 8) {
-                float v[8];
-    #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = to_c(vr[(c + u) * kTile]);
-    #pragma unroll
-                for (int u = 0; u < 8; ++u) b[u] = fmaf(v[u], cf[c + u], b[u]);
-              }
-    #pragma unroll
-              for (int u = 0; u < 8; ++u)
-                if (c + u < c1) b[u] = fmaf(to_c(vr[(c + u) * kTile]), cf[c + u], b[u]);
-              accf = ((b[0] + b[1]) + (b[2] + b[3])) + ((b[4] + b[5]) + (b[6] + b[7]));
+            double b0 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0;
+            int c = c0;
+            for (; c + 4 <= c1; c += 4) {
+              b0 = fma(to_c(vr[(c + 0) * kTile]), cf[c + 0], b0);
+              b1 = fma(to_c(vr[(c + 1) * kTile]), cf[c + 1], b1);
+              b2 = fma(to_c(vr[(c + 2) * kTile]), cf[c + 2], b2);
+              b3 = fma(to_c(vr[(c + 3) * kTile]), cf[c + 3], b3);
             }
-            if (G > 1) {
-              if constexpr (kFp64) comb[g * RS + row] = accd;
-              else reinterpret_cast<float *>(comb)[g * RS + row] = accf;
-            } else {
-              // finish the row here
-              const int64_t r = r0 + row;
-              C base;
-              if (base_bulk) base = to_c(bs[row]);
-              else base = (r < a.n) ? C(to_c(bg[r])) : C(0);
-              if constexpr (MODE == PASS_FIRST) {
-                nrm_add(base * base);
-              } else {
-                const C acc = kFp64 ? C(accd) : C(accf);
-                const C wc = (MODE == PASS_A) ? (base - acc) * C(cscale) : (base - acc);
-                static_cast<C *>(a.w)[r] = wc;
-                ws[row] = wc;
-                if constexpr (MODE == PASS_A) nrm_add(base * base);
-                else if constexpr (MODE == PASS_C || MODE == PASS_B2) nrm_add(wc * wc);
-              }
-            }
+            for (; c < c1; ++c) b0 = fma(to_c(vr[c * kTile]), cf[c], b0);
+            const double accd = (b0 + b1) + (b2 + b3);
+            if (G > 1) comb[g * RS + row] = accd;
+            else finish_row(row, accd);
           }
         }
         if (G > 1) {
           named_bar_sync(1, kConsumers);
           if (tid < RS) {
-            const int row = tid;
             C acc = C(0);
-            if constexpr (kFp64) {
-              for (int g = 0; g < G; ++g) acc += comb[g * RS + row];
-            } else {
-              const float *cb = reinterpret_cast<const float *>(comb);
-              for (int g = 0; g < G; ++g) acc += cb[g * RS + row];
-            }
-            const int64_t r = r0 + row;
-            C base;
-            if (base_bulk) base = to_c(bs[row]);
-            else base = (r < a.n) ? C(to_c(bg[r])) : C(0);
-            const C wc = (MODE == PASS_A) ? (base - acc) * C(cscale) : (base - acc);
-            static_cast<C *>(a.w)[r] = wc;
-            ws[row] = wc;
-            if constexpr (MODE == PASS_A) nrm_add(base * base);
-            else if constexpr (MODE == PASS_C || MODE == PASS_B2) nrm_add(wc * wc);
+            for (int g = 0; g < G; ++g) acc += comb[g * RS + tid];
+            finish_row(tid, acc);
           }
         }
-
       } else {
         // FP32 / BF16 storage: a thread owns a pair of adjacent rows (one 8-byte or 4-byte load
         // gives both) and a group of columns; coefficients come as 16-byte broadcasts (cf is
