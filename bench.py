@@ -351,7 +351,7 @@ def main():
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak if achieved else None,
             "traffic": (ratio * pass_bytes / pass_launches) if (ratio and pass_launches) else None,
-            "kernel": ("streaming passes over V: pass_fused_kernel (A, B, C); pass_ws_kernel (A, B) and pass_kernel (C) where tuned so" if args.reorth == 1 else
+            "kernel": ("streaming passes over V: pass_fused_kernel or pass_ws_kernel (A, B) + pass_kernel (C)" if args.reorth == 1 else
                        "streaming passes over V: lag_fused_kernel or lag_ws_kernel (A2) + pass_fused_kernel or pass_ws_kernel (B2)"),
             "algorithmic_bytes_per_launch": pass_bytes / pass_launches if pass_launches else None,
             "avg_launch_ms": pass_ms / pass_launches if pass_launches else None,

@@ -259,7 +259,7 @@ int foa_dmd_load(const char *path, const foa_dmd_opts *opts, foa_dmd_t **out);
  *             zero-initialised once; on return it holds the unnormalised new direction;
  *   info:     host, result of the push (q after the push, h_last, status).
  * Limits: k_max <= 512 (384 for FP64); the scratch array holds the partial sums of at most 1024
- * CTAs (about 4.8 MB, kept by every GPU that loads the library until the process exits).
+ * CTAs (about 4.5 MB, kept by every GPU that loads the library until the process exits).
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress) and
  * should therefore come before any stream capture.  Every call shares the array and clears
  * what must start at zero; calls that overlap on the GPU (different streams or threads) race

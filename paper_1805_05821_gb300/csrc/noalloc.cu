@@ -23,7 +23,7 @@ constexpr size_t kVecBytes = 3 * size_t(kMaxK) * 8;
 constexpr size_t kPartBytes = size_t(kMaxGrid) * (kMaxK + 1) * 8;
 constexpr size_t kGpartBytes = size_t(kGroups) * (kMaxK + 1) * 8;
 constexpr size_t kCountBytes = 1024;
-constexpr size_t kScratchBytes = kStateBytes + kVecBytes + kPartBytes + kGpartBytes + kCountBytes;  // ~4.8 MB
+constexpr size_t kScratchBytes = kStateBytes + kVecBytes + kPartBytes + kGpartBytes + kCountBytes;  // 4.5 MB
 
 // The scratch shared by every call on a device (held until the process exits).
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];

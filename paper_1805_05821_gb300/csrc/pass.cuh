@@ -18,12 +18,12 @@
 //   sweep 1 (row-local GEMV-N): the new w of every row of the stage;
 //   sweep 2 (GEMV-T split over rows): the column dots, one register accumulator per owned column,
 //           folded into FP64 every 32 products per lane.
-// pass_kernel (this file) runs the FP64 passes and PASS_FIRST, with all eight consumer warps on sweep 1
-// and then on sweep 2.  For FP32/BF16 storage passes A, B, C and B2 run in pass_fused_kernel
-// (pass_fused.cuh), which holds the staged block in registers for both sweeps; the autotuner may pick
-// pass_ws_kernel (pass_ws.cuh: the two sweeps on different warps), or stages too wide for registers, for which pass C
-// runs here.  All end in pass_epilogue.  FP64 storage is bound by the FP64 pipes: A and B keep them 79%
-// busy at j = 51, n = 1048576 (C 71%).
+// pass_kernel (this file) runs pass C and PASS_FIRST for every storage type and passes A, B, B2 for
+// FP64 storage, with all eight consumer warps on sweep 1 and then on sweep 2.  For FP32/BF16 storage
+// passes A, B and B2 run in pass_fused_kernel (pass_fused.cuh: stages of one or two tiles, held in
+// registers for both sweeps) or, for narrower bases, in pass_ws_kernel (pass_ws.cuh), which puts the two
+// sweeps on different warps so that they overlap across stages.  All end in pass_epilogue.  FP64 storage is
+// bound by the FP64 pipes: A and B keep them 79% busy at j = 51, n = 1048576 (C 71%).
 //
 // Every wait is bounded; a timeout records FOA_DMD_ETIMEOUT in the device state and the CTA
 // stops waiting (its results are discarded by the host).
