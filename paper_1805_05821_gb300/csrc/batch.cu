@@ -4,7 +4,7 @@
 //
 //   plan_kernel     reads every stream's device state and the caller's pointer array, decides
 //                   which streams push, and cuts each stream's passes into work items of whole
-//                   pipeline stages (128 KB to 2 MB of V, by the stream's own size);
+//                   pipeline stages (128 KB to 8 MB of V, by the stream's own size);
 //   prep_kernel     beta_pre of every active stream (Alg. 1), one CTA per stream;
 //   bpass_kernel    pass A, then pass B, then pass C (pre-vector, CGS2, norm; Alg. 1) of all streams, one
 //                   launch per pass: two CTAs of 256 threads per SM take items from a counter;
@@ -41,14 +41,15 @@ constexpr int kRingBytes = 102400;          // the stage ring of a CTA (two 50 K
 constexpr int kMaxBSlots = 6;
 constexpr int kCf = 640;                    // padded coefficient vector (>= 16 * 32 + 32)
 // V bytes per work item: a share of the stream's own V, within limits, and nothing of the other streams': an item's
-// ends decide where FP32 column sums are folded and how the FP64 ones are grouped, so a stream has the same
-// bits in any company.  The CTAs take items from a counter: a pass ends unevenly by up to one item a CTA,
-// while every item fills the ring anew and writes its partial sums (about 4 us).  ms from creation to
-// states for 48 streams of 16k to 1M values (120 rounds, 1.9 GB of V) / 3 of 60k to 960k / 20 of 20k to 200k:
-//   share 1/96 149.1 / 19.0 / 20.6, 1/64 146.6 / 23.2 / 21.2, 1/128 152.9 / 17.1 / 21.0, 1/32 up to 8 MB
-//   160.4 / 36.7 / 25.4; 8 MB throughout 178.0 / 109.3 / 94.2; by the round's total bytes 145.5 / 19.7 / 23.0.
-constexpr int64_t kItemBytesMax = 2ll << 20, kItemBytesMin = 128ll << 10;
-constexpr int kItemShare = 96;
+// ends decide where FP32 column sums are folded and how the norms' and the FP64 ones are grouped, so a stream has the
+// same bits in any company.  The CTAs take items from a counter: a pass ends unevenly by up to one item a CTA,
+// while every item fills the ring anew and writes its partial sums (about 4 us).  ms from creation to states for
+// 48 streams of 16k to 1M values (120 rounds, 1.9 GB of V) / 3 of 60k to 960k / 20 of 20k to 200k, and
+// snapshots/s of 256 streams of up to 4M values and 400 columns:
+//   share 1/80 147.0 / 21.0 / 20.7, 5657; 1/64 148.3 / 23.2 / 21.2, 5671; 1/96 149.1 / 18.9 / 20.5, 5640;
+//   8 MB throughout 178.0 / 109.3 / 94.2, 5719; by the round's total bytes 145.5 / 19.7 / 23.0, 5718.
+constexpr int64_t kItemBytesMax = 8ll << 20, kItemBytesMin = 128ll << 10;
+constexpr int kItemShare = 80;
 constexpr int kItemStages = 256;            // at most this many stages ...
 constexpr int kStreamItems = 512;           // ... and this many items of one stream (summed by one CTA)
 enum { PH_A = 0, PH_B = 1, PH_C = 2, PH_APP = 3, NPH = 4 };
